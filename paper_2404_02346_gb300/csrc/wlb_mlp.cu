@@ -9,8 +9,9 @@
 // M = 128, N <= 256, K = 16 per instruction) into an FP32 accumulator in
 // tensor memory, completion is signalled through an mbarrier, and the four
 // warps read the accumulator back with tcgen05.ld for a fused epilogue.
-// Weights are kept as FP32 masters (Adam) with BF16 copies in both
-// orientations for the forward and backward products.
+// Weights are kept as FP32 masters (Adam) with BF16 copies in the layouts that
+// the inference kernel, the training step (wlb_mlp_train.cuh) and the
+// layer-by-layer products read.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -219,12 +220,7 @@ struct Gemm {
     float *C;               // mode 0: FP32 store of rows < m_valid, cols < n_valid
     int ldc;
     const float *bias;      // mode 1: z = acc + bias
-    float *Z;               // mode 1: pre-activation (optional), [M][N]
-    __nv_bfloat16 *H, *HT;  // mode 1: gelu(z) as [M][N] and (optional) [N][ldt]
-    const float *Zin;       // mode 2: dz = acc * gelu'(Zin)
-    __nv_bfloat16 *dZ, *dZT;
-    float *db;              // mode 2: column sums of dz (atomic)
-    int ldt;
+    __nv_bfloat16 *H;       // mode 1: gelu(z) as [M][N]
     int *err;
 };
 
@@ -310,21 +306,8 @@ __global__ void __launch_bounds__(128, 1) umma_gemm(Gemm g) {
                 const int n = cb * 16 + e;
                 if (MODE == 0) {
                     if (m < g.m_valid && n < g.n_valid) g.C[(size_t)m * g.ldc + n] = v[e];
-                } else if (MODE == 1) {
-                    const float z = __fadd_rn(v[e], g.bias[n]);
-                    if (g.Z) g.Z[(size_t)m * g.N + n] = z;
-                    const __nv_bfloat16 h = __float2bfloat16_rn(gv[e]);
-                    g.H[(size_t)m * g.N + n] = h;
-                    if (g.HT) g.HT[(size_t)n * g.ldt + m] = h;
                 } else {
-                    const float dz = v[e] * gelu_grad(g.Zin[(size_t)m * g.N + n]);
-                    const __nv_bfloat16 d = __float2bfloat16_rn(dz);
-                    g.dZ[(size_t)m * g.N + n] = d;
-                    g.dZT[(size_t)n * g.ldt + m] = d;
-                    float s = __bfloat162float(d);
-#pragma unroll
-                    for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                    if (lane == 0) atomicAdd(g.db + n, s);
+                    g.H[(size_t)m * g.N + n] = __float2bfloat16_rn(gv[e]);
                 }
             }
         }
@@ -635,50 +618,20 @@ __global__ void pack_stream(const float *__restrict__ w, __nv_bfloat16 *__restri
     out[e] = __float2bfloat16_rn(v);
 }
 
+// ---------------------------------------------------------------- training
+#include "wlb_mlp_train.cuh"
+
 // ---------------------------------------------------------------- small kernels
-// Inputs x (n x 4 FP32, optionally gathered through perm) -> normalised to
-// [-1, 1] by the box [lo, hi], BF16 [B][16] and [16][B] (padding zero).
-__global__ void prep_inputs(const float *__restrict__ x, const float *__restrict__ t, const int *__restrict__ perm,
-                            long long first, int n, int Bp, const float *lo, const float *hi,
-                            __nv_bfloat16 *__restrict__ X0, __nv_bfloat16 *__restrict__ X0T, float *__restrict__ tb) {
+// Inputs x (n x 4 FP32) -> normalised to [-1, 1] by the box [lo, hi], BF16
+// [B][16] (padding zero).
+__global__ void prep_inputs(const float *__restrict__ x, long long first, int n, int Bp, const float *lo,
+                            const float *hi, __nv_bfloat16 *__restrict__ X0) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= Bp) return;
-    const long long src = perm ? perm[first + i] : first + i;
     for (int a = 0; a < kInPad; ++a) {
         float v = 0.0f;
-        if (i < n && a < kIn) v = normalise_input(x[src * kIn + a], lo[a], hi[a]);
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        X0[(size_t)i * kInPad + a] = h;
-        X0T[(size_t)a * Bp + i] = h;
-    }
-    if (tb) tb[i] = (i < n && t) ? t[src] : 0.0f;
-}
-
-// MSE head: y = Y[:,0] + b4; loss += (y - t)^2 / n; dL/dy = 2 (y - t) / n.
-__global__ void loss_head(const float *__restrict__ Y, const float *__restrict__ b4, const float *__restrict__ t,
-                          int n, int Bp, __nv_bfloat16 *__restrict__ dZ4, __nv_bfloat16 *__restrict__ dZ4T,
-                          float *__restrict__ db4, float *__restrict__ loss) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Bp) return;
-    float g = 0.0f, l = 0.0f;
-    if (i < n) {
-        const float d = Y[(size_t)i * kOutPad] + b4[0] - t[i];
-        l = d * d / (float)n;
-        g = 2.0f * d / (float)n;
-    }
-    const __nv_bfloat16 gb = __float2bfloat16_rn(g);
-    for (int a = 0; a < kOutPad; ++a) {
-        dZ4[(size_t)i * kOutPad + a] = a == 0 ? gb : __float2bfloat16_rn(0.0f);
-        dZ4T[(size_t)a * Bp + i] = a == 0 ? gb : __float2bfloat16_rn(0.0f);
-    }
-    float s = __bfloat162float(gb);
-    for (int o = 16; o >= 1; o >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, o);
-        l += __shfl_xor_sync(0xffffffffu, l, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(db4, s);
-        atomicAdd(loss, l);
+        if (i < n && a < kIn) v = normalise_input(x[(first + i) * kIn + a], lo[a], hi[a]);
+        X0[(size_t)i * kInPad + a] = __float2bfloat16_rn(v);
     }
 }
 
@@ -698,37 +651,17 @@ __global__ void predict_head(const float *__restrict__ Y, const float *__restric
     }
 }
 
-// Adam on the FP32 masters (bias-corrected), then nothing else: BF16 copies
-// are refreshed by pack_weights.
-__global__ void adam(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m1,
-                     float *__restrict__ m2, int n, float lr, float c1, float c2) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float a = 0.9f * m1[i] + 0.1f * gi;
-    const float b = 0.999f * m2[i] + 0.001f * gi * gi;
-    m1[i] = a;
-    m2[i] = b;
-    w[i] -= lr * (a * c1) / (sqrtf(b * c2) + 1e-8f);
-}
-
-// BF16 working copies: W1 [256][16], W2, W3 [256][256], W4 [16][256] (padding
-// zero) and the transposes W2^T, W3^T [256][256], W4^T [256][16].
+// BF16 working copies of the layer-by-layer forward: W1 [256][16], W2, W3
+// [256][256], W4 [16][256] (padding zero).
 __global__ void pack_weights(const float *__restrict__ w, __nv_bfloat16 *W1, __nv_bfloat16 *W2, __nv_bfloat16 *W3,
-                             __nv_bfloat16 *W4, __nv_bfloat16 *W2T, __nv_bfloat16 *W3T, __nv_bfloat16 *W4T) {
+                             __nv_bfloat16 *W4) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;  // over 256 x 256
     if (i >= kHid * kHid) return;
     const int r = i / kHid, c = i % kHid;
     W2[i] = __float2bfloat16_rn(w[oW2 + i]);
     W3[i] = __float2bfloat16_rn(w[oW3 + i]);
-    W2T[c * kHid + r] = __float2bfloat16_rn(w[oW2 + i]);
-    W3T[c * kHid + r] = __float2bfloat16_rn(w[oW3 + i]);
     if (c < kInPad) W1[r * kInPad + c] = __float2bfloat16_rn(c < kIn ? w[oW1 + r * kIn + c] : 0.0f);
-    if (r < kOutPad) {
-        const __nv_bfloat16 v = __float2bfloat16_rn(r == 0 ? w[oW4 + c] : 0.0f);
-        W4[r * kHid + c] = v;
-        W4T[c * kOutPad + r] = v;
-    }
+    if (r < kOutPad) W4[r * kHid + c] = __float2bfloat16_rn(r == 0 ? w[oW4 + c] : 0.0f);
 }
 
 size_t a256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -741,12 +674,15 @@ struct wlb_mlp {
     cudaStream_t stream = nullptr;
     void *mem = nullptr;
     float *w = nullptr, *g = nullptr, *m1 = nullptr, *m2 = nullptr;
-    float *lo = nullptr, *hi = nullptr, *loss = nullptr, *tb = nullptr;
-    __nv_bfloat16 *W1, *W2, *W3, *W4, *W2T, *W3T, *W4T;
-    __nv_bfloat16 *X0, *X0T, *H[3], *HT[3], *dZ[3], *dZT[3], *dZ4, *dZ4T;
-    float *Z[3], *Y;
+    float *lo = nullptr, *hi = nullptr, *loss = nullptr;
+    __nv_bfloat16 *W1, *W2, *W3, *W4;  // layer-by-layer forward: weights,
+    __nv_bfloat16 *X0, *H[3];          // inputs and activations
+    float *Y;
+    TrainBuffers train;                // training step (wlb_mlp_train.cuh)
     uint8_t *Wstream = nullptr;  // fused-forward weight stream (kChunks x kSlotBytes)
-    bool stream_stale = true;    // weights changed since the stream was packed
+    // weights changed since each copy was packed
+    bool stream_stale = true, layered_stale = true, train_stale = true;
+    bool train_configured = false;  // the training kernels' shared-memory limits are set
     bool fused = true;           // predict through mlp_forward_fused
     int fused_grid = 0;          // CTAs of the fused forward (SMs x resident CTAs)
     int *err = nullptr, *perm = nullptr;
@@ -788,8 +724,14 @@ Gemm base_gemm(wlb_mlp *m) {
     return g;
 }
 
-// Forward of one padded batch of Bp rows (X0 staged).  keep: store Z and H^T.
-cudaError_t forward(wlb_mlp *m, int Bp, bool keep) {
+// Layer-by-layer forward of one padded batch of Bp rows (X0 staged).
+cudaError_t forward(wlb_mlp *m, int Bp) {
+    if (m->layered_stale) {
+        pack_weights<<<(kHid * kHid + 255) / 256, 256, 0, m->stream>>>(m->w, m->W1, m->W2, m->W3, m->W4);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        m->layered_stale = false;
+    }
     const __nv_bfloat16 *Win[3] = {m->W1, m->W2, m->W3};
     const int Kin[3] = {kInPad, kHid, kHid};
     const float *bias[3] = {m->w + ob1, m->w + ob2, m->w + ob3};
@@ -800,10 +742,7 @@ cudaError_t forward(wlb_mlp *m, int Bp, bool keep) {
         g.B = Win[l]; g.ldb = Kin[l]; g.n_valid = kHid;
         g.M = Bp; g.N = kHid; g.K = Kin[l];
         g.bias = bias[l];
-        g.Z = keep ? m->Z[l] : nullptr;
         g.H = m->H[l];
-        g.HT = keep ? m->HT[l] : nullptr;
-        g.ldt = Bp;
         cudaError_t e = run_gemm<1>(g, m->stream);
         if (e != cudaSuccess) return e;
         A = m->H[l];
@@ -816,60 +755,73 @@ cudaError_t forward(wlb_mlp *m, int Bp, bool keep) {
     return run_gemm<0>(g, m->stream);
 }
 
-// Loss and gradients of one staged batch (n real rows of Bp) into m->g.
-cudaError_t backward(wlb_mlp *m, int n, int Bp) {
-    cudaError_t e = cudaMemsetAsync(m->g, 0, sizeof(float) * kParams, m->stream);
-    if (e != cudaSuccess) return e;
-    if ((e = forward(m, Bp, true)) != cudaSuccess) return e;
-    loss_head<<<(Bp + 127) / 128, 128, 0, m->stream>>>(m->Y, m->w + ob4, m->tb, n, Bp, m->dZ4, m->dZ4T, m->g + ob4,
-                                                        m->loss);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // layer 4: dW4 = dZ4^T H3, dH3 = dZ4 W4 -> dZ3
-    const __nv_bfloat16 *dA = m->dZ4, *dAT = m->dZ4T;
-    int kprev = kOutPad, mrows = 1;
-    const __nv_bfloat16 *WT[3] = {m->W2T, m->W3T, m->W4T};  // W_{l+1}^T for l = 0..2
-    const int gW[4] = {oW1, oW2, oW3, oW4};
-    const int gb[3] = {ob1, ob2, ob3};
-    for (int l = 2; l >= 0; --l) {
-        // weight gradient of layer l+2 (1-based): dW = dA^T . H_l
-        Gemm w = base_gemm(m);
-        w.A = dAT; w.lda = Bp; w.m_valid = mrows;
-        w.B = m->HT[l]; w.ldb = Bp; w.n_valid = kHid;
-        w.M = ((mrows + kTileM - 1) / kTileM) * kTileM; w.N = kHid; w.K = Bp;
-        w.C = m->g + gW[l + 1]; w.ldc = kHid;
-        if ((e = run_gemm<0>(w, m->stream)) != cudaSuccess) return e;
-        // activation gradient: dH_l = dA . W_{l+2}, dZ_l = dH_l * gelu'(Z_l)
-        Gemm d = base_gemm(m);
-        d.A = dA; d.lda = kprev; d.m_valid = Bp;
-        d.B = WT[l]; d.ldb = kprev; d.n_valid = kHid;
-        d.M = Bp; d.N = kHid; d.K = kprev;
-        d.Zin = m->Z[l]; d.dZ = m->dZ[l]; d.dZT = m->dZT[l]; d.db = m->g + gb[l]; d.ldt = Bp;
-        if ((e = run_gemm<2>(d, m->stream)) != cudaSuccess) return e;
-        dA = m->dZ[l];
-        dAT = m->dZT[l];
-        kprev = kHid;
-        mrows = kHid;
+cudaError_t stage(wlb_mlp *m, const float *x, long long first, int n, int Bp) {
+    prep_inputs<<<(Bp + 127) / 128, 128, 0, m->stream>>>(x, first, n, Bp, m->lo, m->hi, m->X0);
+    return cudaGetLastError();
+}
+
+// Every packed copy of the weights is out of date.
+void weights_changed(wlb_mlp *m) { m->stream_stale = m->layered_stale = m->train_stale = true; }
+
+// Launch on the handle's stream with programmatic dependent launch.
+template <typename P>
+cudaError_t launch_dependent(void (*kernel)(P), const P &p, int grid, int threads, int smem, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, p);
+}
+
+// Samples per CTA of train_tiles: 16 while that gives at most one CTA per SM
+// (a batch of 512: 32 CTAs), else 32 (half the weight loads per sample).
+int train_tile(int n) { return (n + 15) / 16 <= kTilesNarrow ? 16 : 32; }
+
+// What the training kernels need before the first step: the packed weights
+// and the kernels' shared-memory limits on the current device.
+cudaError_t prepare_train(wlb_mlp *m) {
+    cudaError_t e;
+    if (!m->train_configured) {
+        if ((e = cudaFuncSetAttribute(train_tiles<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      train_tile_smem<16>())) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(train_tiles<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      train_tile_smem<32>())) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(train_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, kWeightSmem)) !=
+                cudaSuccess)
+            return e;
+        m->train_configured = true;
     }
-    // layer 1: dW1 = dZ1^T . X0 (4 real input columns)
-    Gemm w = base_gemm(m);
-    w.A = m->dZT[0]; w.lda = Bp; w.m_valid = kHid;
-    w.B = m->X0T; w.ldb = Bp; w.n_valid = kIn;
-    w.M = kHid; w.N = kInPad; w.K = Bp;
-    w.C = m->g + oW1; w.ldc = kIn;
-    return run_gemm<0>(w, m->stream);
+    if (m->train_stale) {
+        pack_train<<<(kHid * kHid + 255) / 256, 256, 0, m->stream>>>(m->w, m->train);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        m->train_stale = false;
+    }
+    return cudaSuccess;
 }
 
-cudaError_t stage(wlb_mlp *m, const float *x, const float *t, const int *perm, long long first, int n, int Bp) {
-    prep_inputs<<<(Bp + 127) / 128, 128, 0, m->stream>>>(x, t, perm, first, n, Bp, m->lo, m->hi, m->X0, m->X0T,
-                                                          m->tb);
-    return cudaGetLastError();
-}
-
-cudaError_t repack(wlb_mlp *m) {
-    m->stream_stale = true;
-    pack_weights<<<(kHid * kHid + 255) / 256, 256, 0, m->stream>>>(m->w, m->W1, m->W2, m->W3, m->W4, m->W2T,
-                                                                   m->W3T, m->W4T);
-    return cudaGetLastError();
+// Loss and gradients of samples first .. first + n - 1 (through perm if
+// given): into g when it is non-null, else applied by Adam.
+cudaError_t train_step(wlb_mlp *m, const float *x, const float *t, const int *perm, long long first, int n, float *g,
+                       float lr, float c1, float c2) {
+    // whole blocks of 64 samples, the missing ones zero
+    const int blocks = (n + kChunkB - 1) / kChunkB, nb = train_tile(blocks * kChunkB);
+    TrainTiles a{};
+    a.x = x; a.t = t; a.perm = perm; a.first = first; a.n = n;
+    a.lo = m->lo; a.hi = m->hi; a.w = m->w; a.b = m->train; a.err = m->err;
+    TrainWeights b{};
+    b.b = m->train; b.blocks = blocks;
+    b.w = m->w; b.m1 = m->m1; b.m2 = m->m2; b.g = g; b.loss = m->loss;
+    b.lr = lr; b.c1 = c1; b.c2 = c2; b.err = m->err;
+    cudaError_t e = nb == 16 ? launch_dependent(train_tiles<16>, a, blocks * kChunkB / nb, kTrainThreads, train_tile_smem<16>(), m->stream)
+                             : launch_dependent(train_tiles<32>, a, blocks * kChunkB / nb, kTrainThreads, train_tile_smem<32>(), m->stream);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(train_weights, b, kWeightJobs, kWeightThreads, kWeightSmem, m->stream);
 }
 
 // Whole inference in one launch of the fused kernel (n >= 1).
@@ -958,16 +910,16 @@ wlb_status wlb_mlp_create(int batch_max, const float x_lo[4], const float x_hi[4
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += a256(bytes); return o; };
     const size_t ow = take(4 * kParams), og = take(4 * kParams), om1 = take(4 * kParams), om2 = take(4 * kParams);
-    const size_t olo = take(16), ohi = take(16), oloss = take(4), otb = take(4 * B), oerr = take(4);
+    const size_t olo = take(16), ohi = take(16), oloss = take(4), oerr = take(4);
     const size_t oW1 = take(2 * H * kInPad), oW2 = take(2 * H * H), oW3 = take(2 * H * H), oW4 = take(2 * kOutPad * H);
-    const size_t oW2T = take(2 * H * H), oW3T = take(2 * H * H), oW4T = take(2 * H * kOutPad);
-    const size_t oX0 = take(2 * B * kInPad), oX0T = take(2 * B * kInPad);
-    size_t oH[3], oHT[3], odZ[3], odZT[3], oZ[3];
+    const size_t oX0 = take(2 * B * kInPad), oY = take(4 * B * kOutPad);
+    size_t oH[3], otH[3], otdZ[3];
     for (int l = 0; l < 3; ++l) {
-        oH[l] = take(2 * B * H); oHT[l] = take(2 * B * H); odZ[l] = take(2 * B * H); odZT[l] = take(2 * B * H);
-        oZ[l] = take(4 * B * H);
+        oH[l] = take(2 * B * H); otH[l] = take(2 * B * H); otdZ[l] = take(2 * B * H);
     }
-    const size_t odZ4 = take(2 * B * kOutPad), odZ4T = take(2 * B * kOutPad), oY = take(4 * B * kOutPad);
+    const size_t otW1 = take(kSmallBytes), otW2 = take(2 * H * H), otW3 = take(2 * H * H), otW4 = take(kSmallBytes);
+    const size_t otX0 = take(2 * B * kInPad), otdz4 = take(1024 * ((B + kChunkB - 1) / kChunkB));
+    const size_t otsq = take(4 * B);
     const size_t oWs = take((size_t)kChunks * kSlotBytes);
     cudaError_t e = cudaGetDevice(&m->device);
     if (e == cudaSuccess) e = cudaMalloc(&m->mem, off);
@@ -978,18 +930,20 @@ wlb_status wlb_mlp_create(int batch_max, const float x_lo[4], const float x_hi[4
     }
     char *p = (char *)m->mem;
     m->w = (float *)(p + ow); m->g = (float *)(p + og); m->m1 = (float *)(p + om1); m->m2 = (float *)(p + om2);
-    m->lo = (float *)(p + olo); m->hi = (float *)(p + ohi); m->loss = (float *)(p + oloss); m->tb = (float *)(p + otb);
+    m->lo = (float *)(p + olo); m->hi = (float *)(p + ohi); m->loss = (float *)(p + oloss);
     m->err = (int *)(p + oerr);
     m->W1 = (__nv_bfloat16 *)(p + oW1); m->W2 = (__nv_bfloat16 *)(p + oW2); m->W3 = (__nv_bfloat16 *)(p + oW3);
-    m->W4 = (__nv_bfloat16 *)(p + oW4); m->W2T = (__nv_bfloat16 *)(p + oW2T); m->W3T = (__nv_bfloat16 *)(p + oW3T);
-    m->W4T = (__nv_bfloat16 *)(p + oW4T);
-    m->X0 = (__nv_bfloat16 *)(p + oX0); m->X0T = (__nv_bfloat16 *)(p + oX0T);
+    m->W4 = (__nv_bfloat16 *)(p + oW4);
+    m->X0 = (__nv_bfloat16 *)(p + oX0); m->Y = (float *)(p + oY);
     for (int l = 0; l < 3; ++l) {
-        m->H[l] = (__nv_bfloat16 *)(p + oH[l]); m->HT[l] = (__nv_bfloat16 *)(p + oHT[l]);
-        m->dZ[l] = (__nv_bfloat16 *)(p + odZ[l]); m->dZT[l] = (__nv_bfloat16 *)(p + odZT[l]);
-        m->Z[l] = (float *)(p + oZ[l]);
+        m->H[l] = (__nv_bfloat16 *)(p + oH[l]);
+        m->train.H[l] = (uint8_t *)(p + otH[l]);
+        m->train.dZ[l] = (uint8_t *)(p + otdZ[l]);
     }
-    m->dZ4 = (__nv_bfloat16 *)(p + odZ4); m->dZ4T = (__nv_bfloat16 *)(p + odZ4T); m->Y = (float *)(p + oY);
+    m->train.W1p = (uint8_t *)(p + otW1); m->train.W2p = (uint8_t *)(p + otW2);
+    m->train.W3p = (uint8_t *)(p + otW3); m->train.W4p = (uint8_t *)(p + otW4);
+    m->train.X0 = (uint8_t *)(p + otX0); m->train.dz4 = (uint8_t *)(p + otdz4);
+    m->train.sq = (float *)(p + otsq);
     m->Wstream = (uint8_t *)(p + oWs);
     e = cudaMemsetAsync(m->mem, 0, off, m->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(m->lo, x_lo, 16, cudaMemcpyHostToDevice, m->stream);
@@ -1009,7 +963,7 @@ wlb_status wlb_mlp_set_weights(wlb_mlp *m, const float *w) {
     MLP_CUDA(m, cudaMemsetAsync(m->m1, 0, sizeof(float) * kParams, m->stream), "adam state");
     MLP_CUDA(m, cudaMemsetAsync(m->m2, 0, sizeof(float) * kParams, m->stream), "adam state");
     m->adam_t = 0;
-    MLP_CUDA(m, repack(m), "pack");
+    weights_changed(m);
     MLP_CUDA(m, cudaStreamSynchronize(m->stream), "synchronize");
     return WLB_OK;
 }
@@ -1039,10 +993,9 @@ wlb_status wlb_mlp_get_weights(wlb_mlp *m, float *w) {
 
 wlb_status wlb_mlp_loss_grad(wlb_mlp *m, const float *x, const float *t, int n, float *loss, float *grad) {
     if (!m || !x || !t || n < 1 || n > m->batch_max) return WLB_ERR_ARG;
-    const int Bp = ((n + kTileM - 1) / kTileM) * kTileM;
     MLP_CUDA(m, cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream), "zero loss");
-    MLP_CUDA(m, stage(m, x, t, nullptr, 0, n, Bp), "stage");
-    MLP_CUDA(m, backward(m, n, Bp), "backward");
+    MLP_CUDA(m, prepare_train(m), "pack");
+    MLP_CUDA(m, train_step(m, x, t, nullptr, 0, n, m->g, 0.0f, 0.0f, 0.0f), "gradient");
     wlb_status s = check_err(m);
     if (s != WLB_OK) return s;
     if (loss) MLP_CUDA(m, cudaMemcpy(loss, m->loss, sizeof(float), cudaMemcpyDeviceToHost), "loss");
@@ -1065,7 +1018,7 @@ wlb_status wlb_mlp_train(wlb_mlp *m, const float *x, const float *t, long long n
     uint64_t s = seed;
     const long long nb = n / batch;  // whole batches per epoch
     if (nb < 1) return WLB_ERR_ARG;
-    for (int ep = 0; ep < epochs; ++ep) {
+    auto shuffle = [&] {
         for (long long i = 0; i < n; ++i) perm[(size_t)i] = (int)i;
         for (long long i = n - 1; i > 0; --i) {  // Fisher-Yates
             const long long j = (long long)(splitmix(s) % (uint64_t)(i + 1));
@@ -1073,19 +1026,22 @@ wlb_status wlb_mlp_train(wlb_mlp *m, const float *x, const float *t, long long n
             perm[(size_t)i] = perm[(size_t)j];
             perm[(size_t)j] = tmp;
         }
+    };
+    MLP_CUDA(m, prepare_train(m), "pack");
+    shuffle();
+    for (int ep = 0; ep < epochs; ++ep) {
         MLP_CUDA(m, cudaMemcpyAsync(m->perm, perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, m->stream), "perm");
         MLP_CUDA(m, cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream), "zero loss");
         const float lr_e = lr * std::pow(lr_final / lr, (float)ep / (float)(epochs > 1 ? epochs - 1 : 1));
+        // train_weights refreshes the training copies itself, the others not
+        m->stream_stale = m->layered_stale = true;
         for (long long k = 0; k < nb; ++k) {
-            MLP_CUDA(m, stage(m, x, t, m->perm, k * batch, batch, batch), "stage");
-            MLP_CUDA(m, backward(m, batch, batch), "backward");
             m->adam_t += 1;
             const float c1 = 1.0f / (1.0f - std::pow(0.9f, (float)m->adam_t));
             const float c2 = 1.0f / (1.0f - std::pow(0.999f, (float)m->adam_t));
-            adam<<<(kParams + 255) / 256, 256, 0, m->stream>>>(m->w, m->g, m->m1, m->m2, kParams, lr_e, c1, c2);
-            MLP_CUDA(m, cudaGetLastError(), "adam");
-            MLP_CUDA(m, repack(m), "pack");
+            MLP_CUDA(m, train_step(m, x, t, m->perm, k * batch, batch, nullptr, lr_e, c1, c2), "training step");
         }
+        if (ep + 1 < epochs) shuffle();  // while this epoch runs (its order is on the device)
         float l = 0;
         MLP_CUDA(m, cudaMemcpyAsync(&l, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream), "loss");
         wlb_status st = check_err(m);
@@ -1104,8 +1060,8 @@ wlb_status wlb_mlp_predict(wlb_mlp *m, const float *x, long long n, float *y, un
     for (long long first = 0; first < n; first += m->batch_max) {
         const int cnt = (int)((n - first) < m->batch_max ? (n - first) : m->batch_max);
         const int Bp = ((cnt + kTileM - 1) / kTileM) * kTileM;
-        MLP_CUDA(m, stage(m, x, nullptr, nullptr, first, cnt, Bp), "stage");
-        MLP_CUDA(m, forward(m, Bp, false), "forward");
+        MLP_CUDA(m, stage(m, x, first, cnt, Bp), "stage");
+        MLP_CUDA(m, forward(m, Bp), "forward");
         predict_head<<<(cnt + 255) / 256, 256, 0, m->stream>>>(m->Y, m->w + ob4, x, first, cnt, m->lo, m->hi, y,
                                                                inside);
         MLP_CUDA(m, cudaGetLastError(), "predict head");
