@@ -14,6 +14,7 @@
 #include <new>
 #include <vector>
 
+#include "wlb_force.cuh"
 #include "wlb_handle.cuh"
 #include "wlb_kernels.cuh"
 
@@ -254,7 +255,29 @@ cudaError_t launch_batch_update(int ch, const LatHot *lats, const int *row_lat, 
 
 __global__ void batch_advance_step(long long *step) { *step += 2; }
 
+// One block per lattice: its force (zeros without samples) and error flag,
+// also written to out[5 * lattice .. ] in host memory (512 lattices: one
+// launch where a kernel and two copies per lattice took 6.6 ms).
+__global__ void __launch_bounds__(kForceThreads) batch_force(const BatchLat *__restrict__ lats, double *out) {
+    const BatchLat &L = lats[blockIdx.x];
+    const long long nw = L.n_steps - L.window_begin;
+    if (nw > 0 && L.g.n_surface > 0) {
+        surface_force_block(L.g, L.b.pts, L.b.acc64, 1.0 / (double)nw, L.b.force, L.b.err);
+    } else if (threadIdx.x < 4) {
+        L.b.force[threadIdx.x] = 0.0;
+    }
+    __syncthreads();
+    double *o = out + 5 * (long long)blockIdx.x;
+    if (threadIdx.x < 4) o[threadIdx.x] = L.b.force[threadIdx.x];
+    if (threadIdx.x == 4) *reinterpret_cast<int *>(o + 4) = *L.b.err;
+}
+
 }  // namespace
+
+cudaError_t launch_batch_force(const BatchLat *d_lats, int count, double *out, cudaStream_t s) {
+    batch_force<<<count, kForceThreads, 0, s>>>(d_lats, out);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_batch_advance(long long *step, cudaStream_t s) {
     batch_advance_step<<<1, 1, 0, s>>>(step);
@@ -521,8 +544,7 @@ cudaError_t plan_two(wlb_batch *b, const wlb::BatchTwoKnobs &kn, bool upload_lat
 }
 
 wlb_status batch_setup(wlb_batch *b) {
-    for (int i = 0; i < b->count; ++i)
-        BATCH_CUDA(b, wlb::launch_setup(b->lat[i].g, b->lat[i].b, b->prec, b->stream), "setup kernels");
+    BATCH_CUDA(b, wlb::launch_batch_setup(b->prec, b->lat.data(), b->d_lats, b->count, b->stream), "setup kernels");
     BATCH_CUDA(b, cudaMemsetAsync(b->d_step, 0, sizeof(long long), b->stream), "reset step");
     BATCH_CUDA(b, cudaMemsetAsync(b->d_done, 0, sizeof(unsigned), b->stream), "reset counter");
     return WLB_OK;
@@ -851,19 +873,9 @@ wlb_status wlb_batch_run(wlb_batch *b, double *forces_out) {
     const long long full = b->max_steps / wlb::kGraphSteps, rest = b->max_steps % wlb::kGraphSteps;
     for (long long k = 0; k < full; ++k) BATCH_CUDA(b, cudaGraphLaunch(b->graph, b->stream), "graph launch");
     BATCH_CUDA(b, issue_steps(b, (int)rest, b->threads, b->blocks_per_sm, b->stream), "step kernels");
-    for (int i = 0; i < b->count; ++i) {
-        const BatchLat &L = b->lat[i];
-        const long long nw = L.n_steps - L.window_begin;
-        if (nw > 0 && L.g.n_surface > 0) {
-            BATCH_CUDA(b, wlb::launch_force(L.g, L.b, (double)nw, b->stream), "force kernel");
-        } else {
-            BATCH_CUDA(b, cudaMemsetAsync(L.b.force, 0, 4 * sizeof(double), b->stream), "zero force");
-        }
-        BATCH_CUDA(b, cudaMemcpyAsync(b->host_out + 5 * i, L.b.force, 4 * sizeof(double), cudaMemcpyDeviceToHost,
-                                      b->stream), "force copy");
-        BATCH_CUDA(b, cudaMemcpyAsync(b->host_out + 5 * i + 4, L.b.err, sizeof(int), cudaMemcpyDeviceToHost,
-                                      b->stream), "flag copy");
-    }
+    double *out = nullptr;  // the pinned buffer as the device addresses it
+    BATCH_CUDA(b, cudaHostGetDevicePointer((void **)&out, b->host_out, 0), "result buffer");
+    BATCH_CUDA(b, wlb::launch_batch_force(b->d_lats, b->count, out, b->stream), "force kernel");
     BATCH_CUDA(b, cudaStreamSynchronize(b->stream), "synchronize");
     bool bad = false;
     for (int i = 0; i < b->count; ++i) {

@@ -56,7 +56,7 @@ struct Buffers {
     unsigned long long *hist_n;  // entries recorded (may exceed the capacity; the excess is dropped)
     int *err;              // 1 int: non-finite accumulator seen
     double *ptab;          // n[wave_axis]: incident pressure along the wave axis (setup)
-    double *stage;         // stage_cells * (1 + dim): field read-back staging
+    double *stage;         // stage_cells * (1 + dim): field read-back staging; tables of the setup
     long long stage_cells;
 };
 
@@ -125,6 +125,14 @@ struct BatchLat {
     long long n_steps, window_begin, period;
     TwoStepPlan plan;
 };
+
+// The setup (launch_setup) of all lattices of a batch in three launches; lats
+// and d_lats are the same descriptors on the host and on the device.
+cudaError_t launch_batch_setup(Prec p, const BatchLat *lats, const BatchLat *d_lats, int count, cudaStream_t s);
+// Forces of all lattices of a batch in one launch (wlb_batch.cu's run): out
+// (device-accessible) gets 4 doubles and the error flag per lattice; zeros
+// for lattices without samples.
+cudaError_t launch_batch_force(const BatchLat *d_lats, int count, double *out, cudaStream_t s);
 
 // Batched two steps per launch (3D): lattices are grouped by lane layout
 // (chunks per lane), one launch of the slab kernel per group.

@@ -18,6 +18,7 @@
 // f / p_a); the scale only enters the setup, the fold and the read-back.
 #include <cmath>
 
+#include "wlb_force.cuh"
 #include "wlb_kernels.cuh"
 
 namespace wlb {
@@ -196,36 +197,11 @@ __global__ void fold_sums(int n, R *__restrict__ acc, double *__restrict__ acc64
     if (!isfinite(v)) atomicExch(err, 1);
 }
 
-// Eq. (14) on the surface elements; one block, fixed reduction order.
-__global__ void __launch_bounds__(256) surface_force(Geometry g, const double *__restrict__ pts,
-                                                     const double *__restrict__ acc64, double inv_nw,
-                                                     double *__restrict__ force, int *__restrict__ err) {
-    __shared__ double red[3][256];
-    const int t = threadIdx.x;
-    double F[3] = {0.0, 0.0, 0.0};
-    const double rho0 = g.rho0;
-    const double inv_2rc2 = 1.0 / (2.0 * rho0 * g.c0 * g.c0);
-    for (int k = t; k < g.n_surface; k += blockDim.x) {
-        const double *row = pts + 7 * (long long)k;
-        const double *a = acc64 + 5 * (long long)k;
-        const double iso = a[0] * inv_nw * inv_2rc2 - 0.5 * rho0 * (a[1] * inv_nw);
-        for (int i = 0; i < 3; ++i) F[i] -= row[6] * (iso * row[3 + i] + rho0 * (a[2 + i] * inv_nw));
-    }
-    for (int i = 0; i < 3; ++i) red[i][t] = F[i];
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (t < s)
-            for (int i = 0; i < 3; ++i) red[i][t] += red[i][t + s];
-        __syncthreads();
-    }
-    if (t == 0) {
-        for (int i = 0; i < 3; ++i) {
-            const double v = i < g.dim ? red[i][0] : 0.0;
-            force[i] = v;
-            if (!isfinite(v)) atomicExch(err, 1);
-        }
-        force[3] = 0.0;
-    }
+// One block (wlb_force.cuh).
+__global__ void __launch_bounds__(kForceThreads) surface_force(Geometry g, const double *__restrict__ pts,
+                                                               const double *__restrict__ acc64, double inv_nw,
+                                                               double *__restrict__ force, int *__restrict__ err) {
+    surface_force_block(g, pts, acc64, inv_nw, force, err);
 }
 
 template <typename S>
@@ -397,7 +373,7 @@ cudaError_t launch_fold(const Geometry &g, const Buffers &b, Prec p, cudaStream_
 }
 
 cudaError_t launch_force(const Geometry &g, const Buffers &b, double n_window, cudaStream_t s) {
-    surface_force<<<1, 256, 0, s>>>(g, b.pts, b.acc64, 1.0 / n_window, b.force, b.err);
+    surface_force<<<1, kForceThreads, 0, s>>>(g, b.pts, b.acc64, 1.0 / n_window, b.force, b.err);
     return cudaGetLastError();
 }
 
