@@ -137,7 +137,9 @@ typedef struct {
     int vector_path;            /* 1 if the row-vectorised update kernel is used */
     int steps_per_launch;       /* steps per update launch: 1, or 2 with
                                    wlb_set_two_step (the default for 3D
-                                   lattices where it applies)                   */
+                                   lattices where it applies); 2D lattices
+                                   that report 1 may still take several per
+                                   launch (see wlb_step)                        */
     int two_step_rows;          /* slab height of the two-step kernel, 0 off    */
     int two_step_segments;      /* warps per lattice row (per x-tile) in it, 0 off */
     int two_step_tiles;         /* x-tiles per row in it (1: whole rows), 0 off */
@@ -177,8 +179,10 @@ wlb_status wlb_init(wlb_handle *h);
  * before its collision, the surface interpolation and the running sums of
  * p1^2, u1.u1 and (n.u1) u1 (Eqs. 80-82); FP32 running sums (FP64 with
  * WLB_POP_F64) are folded into FP64 once per period.  Whole periods are
- * replayed as CUDA graphs captured on first use.  WLB_ERR_STATE before
- * wlb_init. */
+ * replayed as CUDA graphs captured on first use.  On 2D lattices a launch may
+ * take up to eight steps of overlapped tiles, where that is estimated faster
+ * than one (periodic or driven, any row length; bit-identical).
+ * WLB_ERR_STATE before wlb_init. */
 wlb_status wlb_step(wlb_handle *h, long long n_steps, int sample);
 
 /* Time-averaged force from the samples taken since wlb_init, Eq. (14) in
@@ -463,10 +467,11 @@ wlb_status wlb_get_info(const wlb_handle *h, wlb_info *out);
  * 2D lattices (periodic, any storage, rows of at most two 16-byte chunks
  * per lane and 8 values per lane) take it on request (off by default: a
  * single lattice of such short rows has too few row chunks to fill the SMs
- * and one step per launch is faster; 2D batches use it by default): each
+ * and the tiles of wlb_step are faster; 2D batches use it by default): each
  * warp sweeps a chunk of rows, both steps in its registers (slab_rows must
  * be 0).
- * Elsewhere, or with enable = 0, every step is one launch.  enable: 0 off;
+ * Elsewhere, or with enable = 0, 3D steps are one launch each and 2D steps
+ * are those of wlb_step.  enable: 0 off;
  * 1 on, lane layout chosen by the library; 2 on with one 16-byte chunk per
  * lane (more, lighter warps); 3 on with two (WLB_ERR_ARG if unsupported).
  * slab_rows: 0 lets the library choose (by estimated time: slab height and

@@ -161,15 +161,26 @@ bool two_step_plan(const wlb_handle *h, int slab_rows, int mode, int tiles, int 
     return true;
 }
 
+// Steps per launch of the 2D tile kernel, 0 where it is not used.
+int tile_steps(const wlb_handle *h, bool sampled) { return h->two_step ? 0 : h->tile[sampled ? 1 : 0].k; }
+
 // Update launches in one period: each flips the population buffer.
-long long period_launches(const wlb_handle *h, bool) {
-    return h->two_step ? h->period / 2 + h->period % 2 : h->period;
+long long period_launches(const wlb_handle *h, bool sampled) {
+    const int k = h->two_step ? 2 : tile_steps(h, sampled);
+    return k > 0 ? (h->period + k - 1) / k : h->period;
 }
 
 // Issue one period of steps starting from buffer `start` on stream s.
 cudaError_t issue_period(wlb_handle *h, int start, bool sampled, cudaStream_t s) {
     int cur = start;
     long long t = 0;
+    if (const int k = tile_steps(h, sampled))
+        for (; t < h->period; cur ^= 1) {
+            const int n = (int)(h->period - t < k ? h->period - t : k);
+            cudaError_t e = wlb::launch_tile_2d(h->g, h->b, h->prec, h->tile[sampled ? 1 : 0], cur, sampled, n, t, s);
+            if (e != cudaSuccess) return e;
+            t += n;
+        }
     if (h->two_step)
         for (; t + 1 < h->period; t += 2) {  // two steps per launch
             cudaError_t e = two_steps(h, cur, sampled, s);
@@ -331,6 +342,8 @@ wlb_status wlb_create(const wlb_params *p, void *device_workspace, size_t worksp
             h->two_step = true;
             h->two_mode = 1;
         }
+    } else if (wlb::plan_tile_2d(h->g, h->prec, h->tile) != cudaSuccess) {
+        h->tile[0] = h->tile[1] = wlb::TilePlan2D{};  // one step per launch
     }
     cudaGetLastError();
     *out = h;
@@ -366,36 +379,33 @@ wlb_status wlb_step(wlb_handle *h, long long n, int sample) {
             n -= h->period;
             continue;
         }
-        if (h->two_step && n >= 2 && (!sampled || h->samples_in_period + 2 <= h->period)) {
-            WLB_CUDA(h, two_steps(h, h->src, sampled, h->stream),
-                     "two-step kernels");
-            h->src ^= 1;
-            h->steps_done += 2;
-            n -= 2;
-            if (sampled) {
-                h->samples_done += 2;
-                h->samples_in_period += 2;
-                if (h->samples_in_period == h->period) {
-                    WLB_CUDA(h, wlb::launch_fold(h->g, h->b, h->prec, h->stream), "fold kernel");
-                    WLB_CUDA(h, wlb::launch_record_fold(h->g, h->b, h->period, h->stream), "history kernels");
-                    h->samples_in_period = 0;
-                }
-            }
-            continue;
+        // one launch; a sampled one never crosses a period fold
+        const long long room = sampled && h->period - h->samples_in_period < n ? h->period - h->samples_in_period : n;
+        int did = 1;
+        if (h->two_step && room >= 2) {
+            did = 2;
+            WLB_CUDA(h, two_steps(h, h->src, sampled, h->stream), "two-step kernels");
+        } else if (const int k = tile_steps(h, sampled)) {
+            did = (int)(room < k ? room : k);
+            WLB_CUDA(h, wlb::launch_tile_2d(h->g, h->b, h->prec, h->tile[sampled ? 1 : 0], h->src, sampled, did,
+                                            h->steps_done % h->period, h->stream),
+                     "tile kernel");
+        } else {
+            WLB_CUDA(h, wlb::launch_step(h->g, h->b, h->prec, h->src, sampled, h->steps_done % h->period, h->stream),
+                     "step kernels");
         }
-        WLB_CUDA(h, wlb::launch_step(h->g, h->b, h->prec, h->src, sampled, h->steps_done % h->period, h->stream),
-                 "step kernels");
         h->src ^= 1;
-        h->steps_done += 1;
+        h->steps_done += did;
+        n -= did;
         if (sampled) {
-            h->samples_done += 1;
-            if (++h->samples_in_period == h->period) {
+            h->samples_done += did;
+            h->samples_in_period += did;
+            if (h->samples_in_period == h->period) {
                 WLB_CUDA(h, wlb::launch_fold(h->g, h->b, h->prec, h->stream), "fold kernel");
                 WLB_CUDA(h, wlb::launch_record_fold(h->g, h->b, h->period, h->stream), "history kernels");
                 h->samples_in_period = 0;
             }
         }
-        n -= 1;
     }
     return WLB_OK;
 }

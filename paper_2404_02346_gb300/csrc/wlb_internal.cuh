@@ -181,6 +181,25 @@ cudaError_t plan_two_steps_2d(const Geometry &g, Prec p, TwoStepPlan *out);
 cudaError_t launch_two_steps_2d(const Geometry &g, const Buffers &b, Prec p, const TwoStepPlan &pl, int src,
                                 bool sample, cudaStream_t s);
 
+// Several steps per launch for a single 2D lattice (wlb_tile_2d.cu): overlapped
+// tiles of tx x ty cells, up to k steps per launch; k = 0: not used.
+constexpr int kMaxTileSteps = 8;
+struct TilePlan2D {
+    int k = 0, tx = 0, ty = 0, sms = 1;
+    int group = 1;  // surface points per sampler CTA (sampled launches)
+    size_t smem = 0;
+};
+// out[0] for unsampled, out[1] for sampled launches.
+cudaError_t plan_tile_2d(const Geometry &g, Prec p, TilePlan2D out[2]);
+// k <= pl.k steps from buffer src into src ^ 1, the first at step index t_mod of
+// the period; with sample (and pl the sampled plan) the surface sums of all of
+// them are added.
+cudaError_t launch_tile_2d(const Geometry &g, const Buffers &b, Prec p, const TilePlan2D &pl, int src, bool sample,
+                           int k, long long t_mod, cudaStream_t s);
+// rho1 imposed on the driven cavity's source sheet (Eq. 72) at step t_mod of
+// the period, in stored units.
+double source_density(const Geometry &g, long long t_mod);
+
 // The same for batches of 2D lattices (wlb_two_step_2d.cu): a warp sweeps a
 // chunk of rows of one lattice.  Plans every lattice (plan.zc rows per chunk,
 // plan.chunks chunks; rows > 0 fixes plan.zc, else it is chosen to fill whole

@@ -232,9 +232,7 @@ __global__ void read_fields(Geometry g, const S *__restrict__ src, const uint8_t
 template <typename R>
 Drive<R> drive_of(const Geometry &g, long long t_mod) {
     Drive<R> d;
-    const double two_pi = 6.283185307179586476925286766559;
-    d.rho_src = (R)(g.driven ? g.source_amplitude * std::sin(two_pi * (double)t_mod / (double)g.period) * g.pop_scale
-                             : 0.0);
+    d.rho_src = (R)(g.driven ? source_density(g, t_mod) : 0.0);
     d.phi = (R)g.wall_damping;
     d.axis = g.wave_axis;
     return d;
@@ -316,6 +314,11 @@ cudaError_t fields_for(const Geometry &g, const Buffers &b, int src, long long f
 }
 
 }  // namespace
+
+double source_density(const Geometry &g, long long t_mod) {
+    const double two_pi = 6.283185307179586476925286766559;
+    return g.source_amplitude * std::sin(two_pi * (double)t_mod / (double)g.period) * g.pop_scale;
+}
 
 bool update_is_vectorised(const Geometry &g, Prec p) {
     switch (p) {
