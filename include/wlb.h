@@ -137,9 +137,9 @@ typedef struct {
     int vector_path;            /* 1 if the row-vectorised update kernel is used */
     int steps_per_launch;       /* steps per update launch: 1, or 2 with
                                    wlb_set_two_step (the default for 3D
-                                   lattices where it applies); 2D lattices
-                                   that report 1 may still take several per
-                                   launch (see wlb_step)                        */
+                                   lattices where it applies); lattices that
+                                   report 1 may still take several steps per
+                                   launch in tiles (see wlb_step)               */
     int two_step_rows;          /* slab height of the two-step kernel, 0 off    */
     int two_step_segments;      /* warps per lattice row (per x-tile) in it, 0 off */
     int two_step_tiles;         /* x-tiles per row in it (1: whole rows), 0 off */
@@ -181,8 +181,9 @@ wlb_status wlb_init(wlb_handle *h);
  * WLB_POP_F64) are folded into FP64 once per period.  Whole periods are
  * replayed as CUDA graphs captured on first use.  On 2D lattices a launch may
  * take up to eight steps of overlapped tiles, where that is estimated faster
- * than one (periodic or driven, any row length; bit-identical).
- * WLB_ERR_STATE before wlb_init. */
+ * than one (periodic or driven, any row length; bit-identical), and on 3D
+ * lattices without wlb_set_two_step (FP32 and FP16 rows of whole 16-byte
+ * vectors, periodic or driven) two.  WLB_ERR_STATE before wlb_init. */
 wlb_status wlb_step(wlb_handle *h, long long n_steps, int sample);
 
 /* Time-averaged force from the samples taken since wlb_init, Eq. (14) in
@@ -470,8 +471,8 @@ wlb_status wlb_get_info(const wlb_handle *h, wlb_info *out);
  * and the tiles of wlb_step are faster; 2D batches use it by default): each
  * warp sweeps a chunk of rows, both steps in its registers (slab_rows must
  * be 0).
- * Elsewhere, or with enable = 0, 3D steps are one launch each and 2D steps
- * are those of wlb_step.  enable: 0 off;
+ * Elsewhere steps are those of wlb_step; with enable = 0 on a 3D lattice that
+ * takes this kernel every step is one launch.  enable: 0 off;
  * 1 on, lane layout chosen by the library; 2 on with one 16-byte chunk per
  * lane (more, lighter warps); 3 on with two (WLB_ERR_ARG if unsupported).
  * slab_rows: 0 lets the library choose (by estimated time: slab height and

@@ -161,8 +161,21 @@ bool two_step_plan(const wlb_handle *h, int slab_rows, int mode, int tiles, int 
     return true;
 }
 
-// Steps per launch of the 2D tile kernel, 0 where it is not used.
-int tile_steps(const wlb_handle *h, bool sampled) { return h->two_step ? 0 : h->tile[sampled ? 1 : 0].k; }
+// Steps per launch of the tile kernels, 0 where they are not used.
+int tile_steps(const wlb_handle *h, bool sampled) {
+    if (h->two_step) return 0;
+    if (h->g.dim == 2) return h->tile[sampled ? 1 : 0].k;
+    return h->tile3.tx > 0 && (!sampled || h->tile3.boxes > 0) ? 2 : 0;
+}
+
+// One launch of n <= tile_steps(h, sampled) steps from buffer src, the first at
+// index t_mod of the period (3D: one step goes to the one-step kernels).
+cudaError_t tile_launch(wlb_handle *h, int src, bool sampled, int n, long long t_mod, cudaStream_t s) {
+    if (h->g.dim == 2)
+        return wlb::launch_tile_2d(h->g, h->b, h->prec, h->tile[sampled ? 1 : 0], src, sampled, n, t_mod, s);
+    if (n == 1) return wlb::launch_step(h->g, h->b, h->prec, src, sampled, t_mod, s);
+    return wlb::launch_tile_3d(h->g, h->b, h->prec, h->tile3, src, sampled, t_mod, s, h->side);
+}
 
 // Update launches in one period: each flips the population buffer.
 long long period_launches(const wlb_handle *h, bool sampled) {
@@ -177,7 +190,7 @@ cudaError_t issue_period(wlb_handle *h, int start, bool sampled, cudaStream_t s)
     if (const int k = tile_steps(h, sampled))
         for (; t < h->period; cur ^= 1) {
             const int n = (int)(h->period - t < k ? h->period - t : k);
-            cudaError_t e = wlb::launch_tile_2d(h->g, h->b, h->prec, h->tile[sampled ? 1 : 0], cur, sampled, n, t, s);
+            cudaError_t e = tile_launch(h, cur, sampled, n, t, s);
             if (e != cudaSuccess) return e;
             t += n;
         }
@@ -341,6 +354,8 @@ wlb_status wlb_create(const wlb_params *p, void *device_workspace, size_t worksp
         if (two_step_plan(h, 0, 1, 0, 0, 0, &h->two_plan, &pe) && pe == cudaSuccess) {
             h->two_step = true;
             h->two_mode = 1;
+        } else if (wlb::plan_tile_3d(h->g, h->prec, &h->tile3) != cudaSuccess) {
+            h->tile3 = wlb::TilePlan3D{};
         }
     } else if (wlb::plan_tile_2d(h->g, h->prec, h->tile) != cudaSuccess) {
         h->tile[0] = h->tile[1] = wlb::TilePlan2D{};  // one step per launch
@@ -354,6 +369,7 @@ wlb_status wlb_init(wlb_handle *h) {
     if (!h) return WLB_ERR_ARG;
     DeviceGuard dg(h->device);
     WLB_CUDA(h, wlb::launch_setup(h->g, h->b, h->prec, h->stream), "setup kernels");
+    if (h->tile3.boxes > 0) WLB_CUDA(h, wlb::launch_group_points(h->g, h->b, h->stream), "point boxes");
     WLB_CUDA(h, cudaMemsetAsync(h->b.hist_n, 0, sizeof(unsigned long long), h->stream), "history reset");
     h->src = 0;
     h->steps_done = h->samples_done = h->samples_in_period = 0;
@@ -387,9 +403,7 @@ wlb_status wlb_step(wlb_handle *h, long long n, int sample) {
             WLB_CUDA(h, two_steps(h, h->src, sampled, h->stream), "two-step kernels");
         } else if (const int k = tile_steps(h, sampled)) {
             did = (int)(room < k ? room : k);
-            WLB_CUDA(h, wlb::launch_tile_2d(h->g, h->b, h->prec, h->tile[sampled ? 1 : 0], h->src, sampled, did,
-                                            h->steps_done % h->period, h->stream),
-                     "tile kernel");
+            WLB_CUDA(h, tile_launch(h, h->src, sampled, did, h->steps_done % h->period, h->stream), "tile kernels");
         } else {
             WLB_CUDA(h, wlb::launch_step(h->g, h->b, h->prec, h->src, sampled, h->steps_done % h->period, h->stream),
                      "step kernels");

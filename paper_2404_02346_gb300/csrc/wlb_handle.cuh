@@ -31,6 +31,7 @@ struct wlb_handle {
     wlb::TwoStepPlan two_plan;  // its grid, set by wlb_set_two_step
     int two_mode = 0, two_rows = 0, two_tiles = 0, two_staging = 0, two_c2 = 0;  // the settings it was planned with
     wlb::TilePlan2D tile[2];    // 2D, without wlb_set_two_step: several steps per launch (unsampled, sampled)
+    wlb::TilePlan3D tile3;      // 3D, without wlb_set_two_step: two steps per launch in tiles
     wlb::SideStream side;       // sampling beside the two-step update
     double deadline_s = 0.0;    // wlb_run's host-clock limit, 0 = none (wlb_set_deadline)
     cudaEvent_t marks[2] = {nullptr, nullptr};  // period markers of a deadline run

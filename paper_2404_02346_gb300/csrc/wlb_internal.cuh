@@ -44,7 +44,7 @@ struct Buffers {
     uint8_t *band_rows;    // ny * nz: 1 where row (y, z) holds an interface-band cell
     void *c2;              // ncell reals: sound speed squared (read for band cells)
     double *pts;           // n_surface * 7
-    int4 *st_xyz;          // n_surface * stencil: wrapped cell coordinates
+    int4 *st_xyz;          // n_surface * stencil: wrapped cell coordinates (w: grouping of the points, wlb_tile_3d.cu)
     void *st_w;            // n_surface * stencil * 2 reals: (delta c^2, delta / rho0)
     void *nrm;             // n_surface * 4 reals: normal (x, y, z, 0)
     void *acc;             // n_surface * 5 reals: running sums within a period
@@ -67,7 +67,7 @@ cudaError_t launch_update(const Geometry &g, const Buffers &b, Prec p, int src, 
                           bool *vector_path);
 cudaError_t launch_sample(const Geometry &g, const Buffers &b, Prec p, int src, cudaStream_t s);
 // One whole step: the update, plus the surface sampling of the same input when
-// sample is set (fused into the update launch on the row-vectorised path).
+// sample is set (extra blocks of the same launch).
 cudaError_t launch_step(const Geometry &g, const Buffers &b, Prec p, int src, bool sample, long long t_mod,
                         cudaStream_t s);
 cudaError_t launch_fold(const Geometry &g, const Buffers &b, Prec p, cudaStream_t s);
@@ -196,6 +196,20 @@ cudaError_t plan_tile_2d(const Geometry &g, Prec p, TilePlan2D out[2]);
 // them are added.
 cudaError_t launch_tile_2d(const Geometry &g, const Buffers &b, Prec p, const TilePlan2D &pl, int src, bool sample,
                            int k, long long t_mod, cudaStream_t s);
+// Two steps per launch for a single 3D lattice that plan_two_steps does not take
+// (wlb_tile_3d.cu): tiles of tx x ty x tz cells (tx = 0: not used); boxes: grid of
+// the sampling kernel, 0 where sampled steps go one per launch.
+struct TilePlan3D {
+    int tx = 0, ty = 0, tz = 0, threads = 0, boxes = 0;
+    size_t smem = 0;
+};
+cudaError_t plan_tile_3d(const Geometry &g, Prec p, TilePlan3D *out);
+// From buffer src into src ^ 1, the first step at index t_mod of the period; with
+// sample (pl.boxes > 0, launch_group_points after the setup) both steps' surface
+// sums are added beside the update (forked onto side.stream when set).
+cudaError_t launch_tile_3d(const Geometry &g, const Buffers &b, Prec p, const TilePlan3D &pl, int src, bool sample,
+                           long long t_mod, cudaStream_t s, const SideStream &side);
+cudaError_t launch_group_points(const Geometry &g, const Buffers &b, cudaStream_t s);
 // rho1 imposed on the driven cavity's source sheet (Eq. 72) at step t_mod of
 // the period, in stored units.
 double source_density(const Geometry &g, long long t_mod);

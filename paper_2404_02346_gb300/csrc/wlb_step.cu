@@ -143,22 +143,43 @@ __global__ void __launch_bounds__(256) update_rows(const S *__restrict__ src, S 
     }
 }
 
-// Any lattice shape: one thread per cell, scalar accesses.
+// Any lattice shape: one thread per cell, scalar accesses.  As in update_rows,
+// blocks at or beyond cell_blocks sample the surface, and the launch is a
+// programmatic dependent one; with 32-bit index divisions, 64 x 64 x 203 driven
+// FP32 7.5 -> 6.2 us per step, and with 1000 points (a launch of their own before)
+// 10.2 -> 8.2; 57 x 45 x 64 FP32 with 500 points 5.1 -> 3.6.
 template <typename S, int D, bool DRIVEN>
 __global__ void __launch_bounds__(256) update_cells(const S *__restrict__ src, S *__restrict__ dst,
                                                     const uint8_t *__restrict__ cls,
                                                     const typename Store<S>::R *__restrict__ c2f, int nx,
                                                     int ny, int nz, long long ncell,
                                                     typename Store<S>::R c0sq, typename Store<S>::R cpsq,
+                                                    long long cell_blocks, SampleArgs<S> sa,
                                                     Drive<typename Store<S>::R> drv) {
     using R = typename Store<S>::R;
     constexpr int Q = 2 * D + 1;
+    asm volatile("griddepcontrol.launch_dependents;");
+    if ((long long)blockIdx.x >= cell_blocks) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        const int k = (int)((((long long)blockIdx.x - cell_blocks) * blockDim.x + threadIdx.x) >> 5);
+        if (k < sa.g.n_surface) sample_point(sa, src, k, threadIdx.x & 31);
+        return;
+    }
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    int x, y, z;
+    if (ncell <= 0x7fffffffLL) {  // the usual case: 32-bit divisions
+        const unsigned r = (unsigned)id / (unsigned)nx;
+        x = (int)((unsigned)id - r * (unsigned)nx);
+        z = (int)(r / (unsigned)ny);
+        y = (int)(r - (unsigned)z * (unsigned)ny);
+    } else {
+        const long long r = id / nx;
+        x = (int)(id - r * nx);
+        z = (int)(r / ny);
+        y = (int)(r - (long long)z * ny);
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (id >= ncell) return;
-    const int x = (int)(id % nx);
-    const long long r = id / nx;
-    const int y = (int)(r % ny);
-    const int z = (int)(r / ny);
     const long long row = id - x;
     const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
     const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
@@ -238,21 +259,30 @@ Drive<R> drive_of(const Geometry &g, long long t_mod) {
     return d;
 }
 
+// Blocks of 256 threads with programmatic dependent launch, and the blocks that
+// sample the surface (a warp per point).
+cudaLaunchConfig_t dependent_launch(long long blocks, cudaStream_t s, cudaLaunchAttribute (&attr)[1]) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+long long sample_blocks(const Geometry &g, bool sample) {
+    return sample && g.n_surface > 0 ? (g.n_surface + 7) / 8 : 0;
+}
+
 template <typename S, int D, int CH>
 cudaError_t run_rows(const Geometry &g, const Buffers &b, int src, bool sample, long long t_mod, cudaStream_t s) {
     using R = typename Store<S>::R;
     const long long rows = (long long)g.n[1] * g.n[2];
     const long long row_blocks = (rows * 32 + 255) / 256;
-    const long long sample_blocks = sample && g.n_surface > 0 ? (g.n_surface + 7) / 8 : 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(row_blocks + sample_blocks));
-    cfg.blockDim = dim3(256);
-    cfg.stream = s;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cudaLaunchConfig_t cfg = dependent_launch(row_blocks + sample_blocks(g, sample), s, attr);
     auto kern = g.driven ? update_rows<S, D, CH, true> : update_rows<S, D, CH, false>;
     return cudaLaunchKernelEx(&cfg, kern, (const S *)b.pop[src], (S *)b.pop[src ^ 1],
                               (const uint8_t *)b.cls, (const R *)b.c2, g.n[0], g.n[1], g.n[2], g.ncell,
@@ -283,10 +313,11 @@ cudaError_t run_update(const Geometry &g, const Buffers &b, int src, bool sample
     }
     const long long blocks = (g.ncell + 255) / 256;
     auto kern = g.driven ? update_cells<S, D, true> : update_cells<S, D, false>;
-    kern<<<(unsigned)blocks, 256, 0, s>>>(
-        (const S *)b.pop[src], (S *)b.pop[src ^ 1], b.cls, (const R *)b.c2, g.n[0], g.n[1], g.n[2],
-        g.ncell, (R)(g.c0 * g.c0), (R)(g.cp * g.cp), drive_of<R>(g, t_mod));
-    return cudaGetLastError();
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = dependent_launch(blocks + sample_blocks(g, sample), s, attr);
+    return cudaLaunchKernelEx(&cfg, kern, (const S *)b.pop[src], (S *)b.pop[src ^ 1], (const uint8_t *)b.cls,
+                              (const R *)b.c2, g.n[0], g.n[1], g.n[2], g.ncell, (R)(g.c0 * g.c0), (R)(g.cp * g.cp),
+                              blocks, sample_args<S>(g, b), drive_of<R>(g, t_mod));
 }
 
 template <typename S>
@@ -343,15 +374,11 @@ cudaError_t launch_update(const Geometry &g, const Buffers &b, Prec p, int src, 
 
 cudaError_t launch_step(const Geometry &g, const Buffers &b, Prec p, int src, bool sample, long long t_mod,
                         cudaStream_t s) {
-    if (!sample || g.n_surface == 0 || !update_is_vectorised(g, p)) {
-        cudaError_t e = sample && g.n_surface > 0 ? launch_sample(g, b, p, src, s) : cudaSuccess;
-        return e == cudaSuccess ? launch_update(g, b, p, src, t_mod, s, nullptr) : e;
-    }
     bool vec = false;
     switch (p) {
-        case Prec::F64: return update_for<double>(g, b, src, true, t_mod, s, &vec);
-        case Prec::F16: return update_for<__half>(g, b, src, true, t_mod, s, &vec);
-        default: return update_for<float>(g, b, src, true, t_mod, s, &vec);
+        case Prec::F64: return update_for<double>(g, b, src, sample, t_mod, s, &vec);
+        case Prec::F16: return update_for<__half>(g, b, src, sample, t_mod, s, &vec);
+        default: return update_for<float>(g, b, src, sample, t_mod, s, &vec);
     }
 }
 
