@@ -43,6 +43,11 @@
 //
 // Both kernels are launched with programmatic dependent launch; every wait is
 // bounded (WLB_ERR_TIMEOUT).
+//
+// Small predictions (forward_small) are the forward half of train_tiles: for up to
+// a few thousand queries the persistent kernel's 128-query tiles keep a few CTAs
+// busy with 34 weight slices each, one after the other.  The same products and
+// roundings give the same bits.
 
 constexpr int kRegionBytes = 65536, kSmallBytes = 8192;
 constexpr int kTrainEpi = 256, kTrainThreads = 288;  // warps 0-7 epilogues, warp 8 copies and products
@@ -67,6 +72,8 @@ struct TrainTiles {
     int n;            // real samples; the rest of the last tile is zero
     const float *lo, *hi, *w;
     TrainBuffers b;
+    float *y;               // forward only: outputs
+    unsigned char *inside;  // and whether the query lies in the box (optional)
     int *err;
 };
 
@@ -78,8 +85,8 @@ constexpr int train_tile_smem() {
     return kHid * NB * 2 + 2 * kSmallBytes + 3 * kRegionBytes + 128;
 }
 
-template <int NB>
-__global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
+template <int NB, bool TRAIN>
+__device__ __forceinline__ void tile_body(const TrainTiles &a) {
     extern __shared__ uint8_t train_raw[];
     // act first: the output product reads 16 groups of 8 rows from it (rows
     // at or beyond NB are other shared memory and give rows nobody reads)
@@ -88,7 +95,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
     uint8_t *region[3] = {sW4 + kSmallBytes, sW4 + kSmallBytes + kRegionBytes, sW4 + kSmallBytes + 2 * kRegionBytes};
     constexpr uint32_t kCols = NB == 16 ? 64 : 128;  // accumulators: 2 x NB, output: 16
     constexpr int kGroups = NB / 8;
-    __shared__ uint64_t full[4], accum, act_ready, region_free, drain;  // full[0..2] regions, [3] W1 and W4
+    __shared__ uint64_t full[4], accum, act_ready, region_free[2], drain;  // full[0..2] regions, [3] W1 and W4
     __shared__ uint32_t tmem_slot;
     __shared__ float s_dz4[NB];
     __shared__ int s_abort_store;
@@ -103,7 +110,8 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
     if (tid == 0) {
         for (int i = 0; i < 4; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&full[i])));
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&accum)));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&region_free)));
+        for (int i = 0; i < 2; ++i)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&region_free[i])));
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&drain)));
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&act_ready)), "r"(kTrainEpi));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -128,7 +136,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
         }
     }
     float target = 0.0f;  // of sample b0 + lane, in warp 0
-    if (warp == 0 && lane < NB && b0 + lane < a.n)
+    if (TRAIN && warp == 0 && lane < NB && b0 + lane < a.n)
         target = a.t[a.perm ? a.perm[a.first + b0 + lane] : a.first + b0 + lane];
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -154,7 +162,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
             load(1, region[1], a.b.W2p + kRegionBytes, kRegionBytes);
             load(2, region[2], a.b.W3p, kRegionBytes);
             bool ok = true;
-            uint32_t ready = 0, acc = 0;
+            uint32_t ready = 0;
             auto wait = [&](uint64_t *bar, uint32_t phase) { ok = ok && mbar_wait_or_abort(bar, phase, s_abort); };
             auto operands = [&]() {  // the epilogue warps have written the next B operand
                 wait(&act_ready, ready);
@@ -186,18 +194,19 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
                              smem_desc(act0, 128, 4096), id_fwd, 0);
                 mma_commit(&accum);
             }
-            acc ^= 1;
             // layer 2
             wait(&full[0], 0);
             operands();
-            if (ok) half_forward(0, region[0]);
+            if (ok) {
+                half_forward(0, region[0]);
+                mma_commit(&region_free[0]);
+            }
             wait(&full[1], 0);
             if (ok) {
                 half_forward(1, region[1]);
                 mma_commit(&accum);
             }
-            wait(&accum, acc);  // region 0 has been read
-            acc ^= 1;
+            wait(&region_free[0], 0);
             if (ok) load(0, region[0], a.b.W3p + kRegionBytes, kRegionBytes);
             // layer 3
             wait(&full[2], 0);
@@ -216,28 +225,30 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
                              smem_desc(smem_addr(sW4) + k * 256, 128, 4096), id_out, k > 0);
                 mma_commit(&accum);
             }
-            // gradient of H2 = W3^T dZ3
-            operands();
-            if (ok) {
-                half_backward(0, region[2]);
-                mma_commit(&region_free);
-                half_backward(1, region[0]);
-                mma_commit(&accum);
-            }
-            wait(&region_free, 0);
-            if (ok) load(2, region[2], a.b.W2p, kRegionBytes);
-            // gradient of H1 = W2^T dZ2
-            operands();
-            wait(&full[2], 1);
-            if (ok) {
-                half_backward(0, region[2]);
-                half_backward(1, region[1]);
-                mma_commit(&accum);
+            if constexpr (TRAIN) {
+                // gradient of H2 = W3^T dZ3
+                operands();
+                if (ok) {
+                    half_backward(0, region[2]);
+                    mma_commit(&region_free[1]);
+                    half_backward(1, region[0]);
+                    mma_commit(&accum);
+                }
+                wait(&region_free[1], 0);
+                if (ok) load(2, region[2], a.b.W2p, kRegionBytes);
+                // gradient of H1 = W2^T dZ2
+                operands();
+                wait(&full[2], 1);
+                if (ok) {
+                    half_backward(0, region[2]);
+                    half_backward(1, region[1]);
+                    mma_commit(&accum);
+                }
             }
             if (!ok) {
                 if (!*s_abort) {
                     *s_abort = 1;
-                    atomicExch(a.err, 1);
+                    raise(a.err);
                 }
                 // copies in flight land before the CTA exits
                 for (int r = 0; r < 4; ++r)
@@ -255,7 +266,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
         const size_t my_out = (size_t)(b0 / kChunkB) * (kHid * kChunkB * 2) + (size_t)(f >> 3) * 1024 +
                               (size_t)((b0 % kChunkB) / 8) * 128 + (size_t)(f & 7) * 16;  // group g at + 128 g
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
+        for (int j = 0; j < (TRAIN ? kPer : 0); ++j) {
             const int e = tid + j * kTrainEpi, k = e / NB, b = b0 + e % NB;
             *reinterpret_cast<__nv_bfloat16 *>(a.b.X0 + (size_t)(b / kChunkB) * (kInPad * kChunkB * 2) +
                                                (k >> 3) * 1024 + ((b % kChunkB) >> 3) * 128 + (k & 7) * 16 +
@@ -274,7 +285,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
             for (int g = 0; g < kGroups; ++g) {
                 const uint4 v = make_uint4(pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
                 if (operand) *reinterpret_cast<uint4 *>(my_act + g * 4096) = v;
-                *reinterpret_cast<uint4 *>(out + my_out + g * 128) = v;
+                if (TRAIN) *reinterpret_cast<uint4 *>(out + my_out + g * 128) = v;
             }
         };
         uint32_t phase = 0;
@@ -293,7 +304,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
                 }
             }
         };
-        float gp[3][NB];
+        float gp[3][TRAIN ? NB : 1];
         publish();
         // no early exit from here: every warp reaches the block barriers and the
         // named barrier below; a failed wait skips the work
@@ -319,10 +330,20 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
                 // ahead of it and holds every layer back by up to 2.7k cycles
                 if (*s_abort) {
                     ok = false;
-                } else {
+                } else if constexpr (TRAIN) {
 #pragma unroll
                     for (int e = 0; e < NB; ++e) gp[l][e] = gelu_grad(v[e]);
                 }
+            }
+        }
+        if constexpr (!TRAIN) {
+            if (warp == 1 && lane < NB && b0 + lane < a.n && a.inside) {
+                bool in = true;
+                for (int e = 0; e < kIn; ++e) {
+                    const float xv = a.x[(size_t)(b0 + lane) * kIn + e];
+                    in &= xv >= a.lo[e] && xv <= a.hi[e];
+                }
+                a.inside[b0 + lane] = in ? 1 : 0;
             }
         }
         // output, loss and dL/dy: one lane of warp 0 per sample
@@ -335,12 +356,13 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
                 tmem_ld16(tmem + 2 * NB, v);
                 const int b = b0 + lane;
                 float g = 0.0f, l = 0.0f;
-                if (lane < NB && b < a.n) {
+                if (!TRAIN && lane < NB && b < a.n) a.y[b] = v[0] + b4;
+                if (TRAIN && lane < NB && b < a.n) {
                     const float d = v[0] + b4 - target;
                     l = d * d / (float)a.n;
                     g = 2.0f * d / (float)a.n;
                 }
-                if (lane < NB) {
+                if (TRAIN && lane < NB) {
                     const __nv_bfloat16 gb = __float2bfloat16_rn(g);
                     s_dz4[lane] = __bfloat162float(gb);
                     *reinterpret_cast<__nv_bfloat16 *>(a.b.dz4 + (size_t)(b / kChunkB) * 1024 +
@@ -349,34 +371,36 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
                 }
             }
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(kTrainEpi) : "memory");
-        const float w4 = __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(sW4 + (f >> 3) * 128 + (f & 7) * 2));
+        if constexpr (TRAIN) {
+            asm volatile("bar.sync 1, %0;" ::"n"(kTrainEpi) : "memory");
+            const float w4 = __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(sW4 + (f >> 3) * 128 + (f & 7) * 2));
 #pragma unroll
-        for (int l = 2; l >= 0; --l) {
-            float v[NB];
-            if (l == 2) {
-                // dH3 = dL/dy W4: the product of two BF16 values is exact
+            for (int l = 2; l >= 0; --l) {
+                float v[NB];
+                if (l == 2) {
+                    // dH3 = dL/dy W4: the product of two BF16 values is exact
 #pragma unroll
-                for (int e = 0; e < NB; ++e) v[e] = s_dz4[e] * w4;
-            } else {
-                accumulator(v);
-            }
-            if (ok) {
-                uint32_t pk[NB / 2];
-#pragma unroll
-                for (int e = 0; e < NB; e += 2) {
-                    __nv_bfloat162 p;
-                    p.x = grad_bf16(v[e], gp[l][e]);
-                    p.y = grad_bf16(v[e + 1], gp[l][e + 1]);
-                    pk[e / 2] = *reinterpret_cast<const uint32_t *>(&p);
+                    for (int e = 0; e < NB; ++e) v[e] = s_dz4[e] * w4;
+                } else {
+                    accumulator(v);
                 }
-                store(pk, a.b.dZ[l], l > 0);
-                if (l > 0) publish();
+                if (ok) {
+                    uint32_t pk[NB / 2];
+#pragma unroll
+                    for (int e = 0; e < NB; e += 2) {
+                        __nv_bfloat162 p;
+                        p.x = grad_bf16(v[e], gp[l][e]);
+                        p.y = grad_bf16(v[e + 1], gp[l][e + 1]);
+                        pk[e / 2] = *reinterpret_cast<const uint32_t *>(&p);
+                    }
+                    store(pk, a.b.dZ[l], l > 0);
+                    if (l > 0) publish();
+                }
             }
         }
         if (!ok && !*s_abort) {
             *s_abort = 1;
-            atomicExch(a.err, 1);
+            raise(a.err);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -385,6 +409,15 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
     }
+}
+
+template <int NB>
+__global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(TrainTiles a) {
+    tile_body<NB, true>(a);
+}
+template <int NB>
+__global__ void __launch_bounds__(kTrainThreads, 1) forward_small(TrainTiles a) {
+    tile_body<NB, false>(a);
 }
 
 struct TrainWeights {
@@ -566,7 +599,7 @@ __global__ void __launch_bounds__(kWeightThreads, 1) train_weights(TrainWeights 
             } else {
                 if (!*s_abort) {
                     *s_abort = 1;
-                    atomicExch(a.err, 1);
+                    raise(a.err);
                 }
                 for (int c = issued > kWSlots ? issued - kWSlots : 0; c < issued; ++c)
                     mbar_wait(&full[c % kWSlots], (uint32_t)((c / kWSlots) & 1));
@@ -649,7 +682,7 @@ __global__ void __launch_bounds__(kWeightThreads, 1) train_weights(TrainWeights 
             }
         } else if (!*s_abort) {
             *s_abort = 1;
-            atomicExch(a.err, 1);
+            raise(a.err);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

@@ -78,3 +78,22 @@ def test_one_training_step_is_adam_on_the_reported_gradient(wlb, batch):
     assert np.array_equal(ga, gb)
     net.close()
     net2.close()
+
+
+@pytest.mark.parametrize("n", [1, 16, 17, 2432, 2433, 9728, 9729])
+def test_small_predictions_equal_the_layered_forward(wlb, n):
+    """Predictions of up to 9728 queries run the forward half of the training
+    tiles (16 or 32 queries per CTA), larger ones the persistent kernel: both
+    give the bits of the layer-by-layer launches, flags included."""
+    import torch
+    x, _ = _inputs(n, n)
+    x[2::5, 0] = 4.0
+    x[3::7, 3] = 0.1
+    xt = torch.tensor(x, dtype=torch.float32, device="cuda")
+    net = wlb.MLP(LO, HI, batch_max=1024)
+    net.init_weights(8)
+    y, inside = net.predict(xt)
+    net.set_fused(False)
+    yl, insl = net.predict(xt)
+    assert torch.equal(y, yl) and torch.equal(inside, insl) and torch.isfinite(y).all()
+    net.close()
