@@ -500,6 +500,10 @@ def run_ensemble(args):
     bpu = 2 * q * size + 1
     cells_all = sum(int(np.prod(p["n"][:p["dim"]])) for p in probs)
     spl = info.steps_per_launch if info.steps_per_launch > 0 else 1
+    rows2d = args.workload == "ensemble2d" and args.precision != "f64" and spl == 2
+    if rows2d:
+        spl = 6           # rows of 192 cells: six steps per launch
+        bpu = 2 * q * size + 4  # and c^2 read in place of the class byte
     launch_ms = tune["ms_per_step"] * spl
     achieved = bpu * cells_all / (launch_ms * 1e-3) / 1e9
     peaks = _peaks()
@@ -517,11 +521,11 @@ def run_ensemble(args):
     traffic = None
     if args.workload == "ensemble3d" and args.precision == "f32" and len(probs) == 64 and spl == 2:
         traffic = _traffic(_kernel_sha(2), name="batch_update2_d3q7_f32_ensemble64.md")
-    elif args.workload == "ensemble2d" and args.precision == "f32" and len(probs) == 512 and spl == 2:
-        traffic = _traffic(_kernel_sha(2, "wlb_two_step_2d.cu"), name="batch2d_update2_d2q5_f32_ensemble512.md")
+    elif rows2d and args.precision == "f32" and len(probs) == 512:
+        traffic = _traffic(_kernel_sha(2, "wlb_batch_2d.cu"), name="batch_rows_2d_d2q5_f32_ensemble512.md")
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "traffic": traffic, "kernel": ("batched two-step update" if spl == 2 else "batched update")
-                                          + " (%s storage), all lattices" % args.precision,
+                "traffic": traffic, "kernel": "batched %supdate (%s storage), all lattices"
+                                          % ({1: "", 2: "two-step ", 6: "six-step "}[spl], args.precision),
                 "bytes_per_cell_per_launch": bpu, "avg_launch_us": launch_ms * 1e3,
                 "peak_source": ("measured" if peaks and "hbm_gbs" in peaks else "fallback") + " hbm_gbs"}
     line = {

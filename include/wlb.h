@@ -365,7 +365,8 @@ typedef struct {
     int threads_per_block, blocks_per_sm, row_chunks;
     int steps_per_launch;           /* 2: every launch advances all lattices two
                                        steps (wlb_set_two_step's kernel, one
-                                       launch over every lattice's slabs)      */
+                                       launch over every lattice's slabs) or
+                                       several (2D, wlb_batch_set_two_step)    */
     int total_ctas;                 /* work units of that launch: blocks (3D)
                                        or warps, one per row chunk (2D); 0 if
                                        one step per launch                    */
@@ -384,8 +385,11 @@ wlb_status wlb_batch_get_info(const wlb_batch *b, wlb_batch_info *out);
  * plan; with two lane layouts the two launches run side by side, the second
  * on a stream the batch creates and joins back into its own) or 2D with
  * rows of at most 64 sixteen-byte vectors and 8 values per lane (then each
- * warp sweeps a chunk of 32 rows of one lattice, both steps in registers).
- * A batched sampling launch adds the sums of both steps.  Bit-identical to
+ * warp sweeps a chunk of rows of one lattice with all steps of the launch in
+ * registers: FP32 and FP16 rows of up to 128 cells eight steps, wider ones six
+ * or four, a period's last launch what is left of it; FP64, and rows of 252
+ * cells, two).
+ * A batched sampling launch adds the sums of all steps.  Bit-identical to
  * one step per launch.  enable = 0 returns to one step per launch;
  * enable != 0 where the batch does not qualify gives WLB_ERR_ARG. */
 wlb_status wlb_batch_set_two_step(wlb_batch *b, int enable);

@@ -320,8 +320,10 @@ struct wlb_batch {
     // counts): one launch of the slab kernel over every lattice's CTAs
     bool two_ok = false, two = false;
     int two_threads = 0, total_ctas = 0;  // 2D: total_ctas counts warps (row chunks)
-    wlb::BatchTwoGroup groups[2];         // 3D: lane-layout groups, one launch each
+    wlb::BatchTwoGroup groups[wlb::kMaxRowGroups];  // lane-layout groups, one launch each (3D, 2D row sweeps)
     int ngroups = 0;
+    bool rows2d = false;                  // 2D FP32/FP16: several steps per launch (wlb_batch_2d.cu)
+    wlb::BatchTurns turns;                // its launches
     int two_ch = 1;                       // 2D: chunks per lane of the widest row
     int two_nx = 0;                       // 2D: widest row (staging slot size)
     int *d_cta_lat = nullptr, *d_cta_first = nullptr;
@@ -395,6 +397,23 @@ wlb_status batch_validate(const wlb_params *ps, int count) {
         if (ps[i].nx % W != 0 || ps[i].nx > 32 * W * wlb::kMaxChunks) return WLB_ERR_ARG;
     }
     return WLB_OK;
+}
+
+// Launches n0 .. n1 - 1 of a run by 2D row sweeps.
+cudaError_t issue_rows(wlb_batch *b, int n0, int n1) {
+    for (int n = n0; n < n1; ++n) {
+        cudaError_t e = wlb::launch_batch2d_rows(b->prec, b->groups, b->ngroups, b->d_lats, b->d_cta_lat,
+                                                 b->d_cta_first, b->count, b->turns, n, b->stream);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// Steps of its longest launches.
+int rows_steps(const wlb_batch *b) {
+    int k = 2;
+    for (const BatchLat &L : b->lat) k = std::max(k, L.plan.nseg);
+    return k;
 }
 
 cudaError_t issue_steps(wlb_batch *b, int nsteps, int threads, int bps, cudaStream_t s) {
@@ -497,26 +516,31 @@ cudaError_t issue_steps(wlb_batch *b, int nsteps, int threads, int bps, cudaStre
 cudaError_t plan_two(wlb_batch *b, const wlb::BatchTwoKnobs &kn, bool upload_lats) {
     const int count = b->count;
     std::vector<BatchLat> lat = b->lat;
-    wlb::BatchTwoGroup groups[2];
+    wlb::BatchTwoGroup groups[wlb::kMaxRowGroups];
     int ngroups = 0, tasks2d = 0, two_ch = b->two_ch, two_nx = b->two_nx;
+    // 2D rows go several steps per launch; FP64, which the FP64 pipe bounds either
+    // way, and rows that leave no room for a halo two (plan_batch2d_rows takes
+    // nothing that plan_batch2d_two_steps would not)
+    const bool rows2d = b->dim == 2 && wlb::plan_batch2d_rows(b->prec, lat.data(), count, kn.rows_2d, groups, &ngroups);
     const bool planned = b->dim == 3 ? wlb::plan_batch_two_steps(b->prec, lat.data(), count, kn, groups, &ngroups)
-                                     : wlb::plan_batch2d_two_steps(b->prec, lat.data(), count, kn.rows_2d, &tasks2d,
-                                                                   &two_ch, &two_nx);
+                                     : rows2d || wlb::plan_batch2d_two_steps(b->prec, lat.data(), count, kn.rows_2d,
+                                                                             &tasks2d, &two_ch, &two_nx);
     if (!planned) return cudaErrorInvalidValue;
     // CTA (3D) or warp (2D) -> lattice table, the lattices of each 3D
     // lane-layout group together; first[i] = lattice i's first entry
     std::vector<int> first(count + 1, 0), owner;
-    const int ngr = b->dim == 3 ? ngroups : 1;
+    const bool grouped = b->dim == 3 || rows2d;
+    const int ngr = grouped ? ngroups : 1;
     int two_threads = 0;
     for (int k = 0; k < ngr; ++k) {
         const int begin = (int)owner.size();
         for (int i = 0; i < count; ++i) {
-            if (b->dim == 3 && lat[i].plan.chunks_per_lane != groups[k].ch) continue;
+            if (grouped && lat[i].plan.chunks_per_lane != groups[k].ch) continue;
             const int n = lat[i].plan.nslab * lat[i].plan.chunks;
             first[i] = (int)owner.size();
             owner.insert(owner.end(), (size_t)n, i);
         }
-        if (b->dim == 3) {
+        if (grouped) {
             groups[k].cta_begin = begin;
             groups[k].ctas = (int)owner.size() - begin;
             two_threads = std::max(two_threads, groups[k].threads);
@@ -532,8 +556,10 @@ cudaError_t plan_two(wlb_batch *b, const wlb::BatchTwoKnobs &kn, bool upload_lat
         e = cudaMemcpy(b->d_lats, lat.data(), sizeof(BatchLat) * count, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
     b->lat = lat;
-    for (int k = 0; k < 2; ++k) b->groups[k] = groups[k];
+    for (int k = 0; k < wlb::kMaxRowGroups; ++k) b->groups[k] = groups[k];
     b->ngroups = ngroups;
+    b->rows2d = rows2d;
+    if (rows2d) b->turns = wlb::batch2d_turns(b->lat.data(), count);
     b->two_ch = two_ch;
     b->two_nx = two_nx;
     b->two_threads = two_threads;
@@ -728,8 +754,18 @@ wlb_status wlb_batch_autotune(wlb_batch *b, int steps_per_trial, wlb_batch_tunin
     if (b->two) {
         // time one plan: a warm-up pair of steps, then steps from step 0 (all
         // lattices active)
-        const int steps = 2 * ((steps_per_trial + 1) / 2);
+        const int per_launch = b->rows2d ? rows_steps(b) : 2;
+        const int launches = (steps_per_trial + per_launch - 1) / per_launch, steps = launches * per_launch;
         auto trial = [&](float *ms) -> cudaError_t {
+            if (b->rows2d) {
+                cudaError_t e = issue_rows(b, 0, 1);
+                if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
+                if (e == cudaSuccess) e = issue_rows(b, 0, launches);
+                if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
+                if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+                if (e == cudaSuccess) e = cudaEventElapsedTime(ms, e0, e1);
+                return e;
+            }
             cudaError_t e = cudaMemsetAsync(b->d_step, 0, sizeof(long long), b->stream);
             if (e == cudaSuccess) e = issue_steps(b, 2, b->threads, b->blocks_per_sm, b->stream);
             if (e == cudaSuccess) e = cudaMemsetAsync(b->d_step, 0, sizeof(long long), b->stream);
@@ -847,7 +883,10 @@ wlb_status wlb_batch_run(wlb_batch *b, double *forces_out) {
     if (!b || !forces_out) return WLB_ERR_ARG;
     wlb_status st = batch_setup(b);
     if (st != WLB_OK) return st;
-    if (!b->graph || b->graph_threads != b->threads || b->graph_bps != b->blocks_per_sm ||
+    if (b->two && b->rows2d) {
+        // the launches know their step: no graph (they are as long as a host launch takes or longer)
+        BATCH_CUDA(b, issue_rows(b, 0, b->turns.launches), "step kernels");
+    } else if (!b->graph || b->graph_threads != b->threads || b->graph_bps != b->blocks_per_sm ||
         b->graph_two != (int)b->two || b->graph_plan_gen != b->plan_gen) {
         if (b->graph) cudaGraphExecDestroy(b->graph);
         b->graph = nullptr;
@@ -870,9 +909,11 @@ wlb_status wlb_batch_run(wlb_batch *b, double *forces_out) {
         b->graph_two = (int)b->two;
         b->graph_plan_gen = b->plan_gen;
     }
-    const long long full = b->max_steps / wlb::kGraphSteps, rest = b->max_steps % wlb::kGraphSteps;
-    for (long long k = 0; k < full; ++k) BATCH_CUDA(b, cudaGraphLaunch(b->graph, b->stream), "graph launch");
-    BATCH_CUDA(b, issue_steps(b, (int)rest, b->threads, b->blocks_per_sm, b->stream), "step kernels");
+    if (!(b->two && b->rows2d)) {
+        const long long full = b->max_steps / wlb::kGraphSteps, rest = b->max_steps % wlb::kGraphSteps;
+        for (long long k = 0; k < full; ++k) BATCH_CUDA(b, cudaGraphLaunch(b->graph, b->stream), "graph launch");
+        BATCH_CUDA(b, issue_steps(b, (int)rest, b->threads, b->blocks_per_sm, b->stream), "step kernels");
+    }
     double *out = nullptr;  // the pinned buffer as the device addresses it
     BATCH_CUDA(b, cudaHostGetDevicePointer((void **)&out, b->host_out, 0), "result buffer");
     BATCH_CUDA(b, wlb::launch_batch_force(b->d_lats, b->count, out, b->stream), "force kernel");

@@ -172,6 +172,25 @@ cudaError_t launch_batch_two_steps(Prec p, const BatchTwoGroup *groups, int ngro
 // when its groups ran side by side.
 cudaError_t launch_batch_advance(long long *step, cudaStream_t s);
 
+// Several steps per launch for batches of 2D lattices (wlb_batch_2d.cu), FP32 and
+// FP16: plans every lattice and fills up to kMaxRowGroups groups, one per number of
+// cells per lane (ch; cta_begin / ctas, here warps, are left to the caller); rows:
+// rows per warp chunk, 0 chooses.  False if some lattice cannot take it.  Periods
+// must be even.
+constexpr int kMaxRowGroups = 7;
+bool plan_batch2d_rows(Prec p, BatchLat *lats, int count, int rows, BatchTwoGroup *groups, int *ngroups);
+// Launches of a run; the first one with samples, its sampler blocks per lattice
+// and the steps of a sampled launch at most.
+struct BatchTurns {
+    int launches = 0, first_sampled = 0, groups = 0, steps = 0;
+};
+BatchTurns batch2d_turns(const BatchLat *lats, int count);
+// Launch n of a run: every lattice that is not done advances by the steps its
+// period has left, plan.nseg at most; the state before it is in buffer n & 1.
+cudaError_t launch_batch2d_rows(Prec p, const BatchTwoGroup *groups, int ngroups, const BatchLat *lats,
+                                const int *task_lat, const int *task_first, int count, const BatchTurns &turns, int n,
+                                cudaStream_t s);
+
 // Two steps per launch for a single 2D lattice (wlb_two_step_2d.cu): periodic,
 // rows of at most two 16-byte chunks (8 values) per lane; each warp sweeps a
 // chunk of plan.zc rows (plan.chunks chunks).  From buffer src into src ^ 1;

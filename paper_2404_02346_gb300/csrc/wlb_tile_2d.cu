@@ -21,21 +21,12 @@
 // FP64 lattices are bound by the FP64 pipe (about two instructions per clock
 // and SM): tiles spread the lattice over all SMs and box cells are numbered
 // linearly so that warps are full.  Figures beside the planner below.
-#include <cmath>
-
-#include "wlb_handle.cuh"
-#include "wlb_kernels.cuh"
+#include "wlb_box_2d.cuh"
 
 namespace wlb {
 namespace {
 
 constexpr int kThreads = 512;   // a box cell each, so that latency is paid about once per step
-constexpr int kMaxGroup = 64;   // points of a sampler CTA (four lanes each)
-constexpr float kMaxArc = 8.0f; // and the length of their arc in cells
-
-// The value a stored state holds for v (storage rounding).
-template <typename S> __device__ __forceinline__ typename Store<S>::R as_stored(typename Store<S>::R v) { return v; }
-template <> __device__ __forceinline__ float as_stored<__half>(float v) { return __half2float(__float2half_rn(v)); }
 
 template <typename S>
 struct TileArgs {
@@ -66,33 +57,6 @@ __host__ __device__ inline size_t box_smem(int w, int h, bool sampler, bool driv
     return (sampler ? 17 : 11) * area * sizeof(R) + (size_t)(w + h) * sizeof(int) + (driven ? area : 0);
 }
 
-// Largest moment box of a sampler CTA, in cells: the arc's extent, one cell of
-// stencil on either side and two of rounding.
-__host__ __device__ constexpr int sampler_box() { return (int)kMaxArc + 5; }
-
-// i / w for 0 <= i < 2^16 and w >= 1 by the high half of a product with
-// ceil(2^32 / w) (which does not fit 32 bits for w = 1: a box one cell wide).
-__device__ __forceinline__ unsigned divide_magic(int w) { return w > 1 ? 0xffffffffu / (unsigned)w + 1u : 0u; }
-__device__ __forceinline__ int divide(int i, int w, unsigned magic) {
-    return w > 1 ? (int)__umulhi((unsigned)i, magic) : i;
-}
-
-// The collision of collide_half for D = 2, with rho1 returned.  2 eq and
-// 2 (rho1 - 2 eq) are exact, so the two fused multiply-adds round exactly as
-// the product and difference do; they save two of thirteen operations, which
-// in FP64 are the kernel's bound.
-template <typename R>
-__device__ __forceinline__ R collide_2d(R c2, const R (&f)[5], R (&o)[5]) {
-    const R rho = add_rn(add_rn(add_rn(add_rn(f[0], f[1]), f[2]), f[3]), f[4]);
-    const R eq = mul_rn(c2, rho);
-    o[0] = fma_rn(R(2), fma_rn(R(-2), eq, rho), -f[0]);
-    o[1] = sub_rn(eq, f[2]);
-    o[2] = sub_rn(eq, f[1]);
-    o[3] = sub_rn(eq, f[4]);
-    o[4] = sub_rn(eq, f[3]);
-    return rho;
-}
-
 template <typename S, bool DRIVEN, bool SAMPLE>
 __global__ void __launch_bounds__(kThreads) tile_steps_2d(TileArgs<S> P) {
     using R = typename Store<S>::R;
@@ -111,30 +75,8 @@ __global__ void __launch_bounds__(kThreads) tile_steps_2d(TileArgs<S> P) {
     int x0, y0, tw, th;
     if (sampler) {
         if (tid < 32) {
-            const int p0 = (int)blockIdx.x * P.group, p1 = min(P.n_surface, p0 + P.group);
-            float lox = 1e30f, hix = -1e30f, loy = 1e30f, hiy = -1e30f;
-            for (int p = p0 + tid; p < p1; p += 32) {
-                float sn, cs;
-                sincospif((float)(2 * p + 1) / (float)P.n_surface, &sn, &cs);
-                const float X = P.cx + P.radius * cs, Y = P.cy + P.radius * sn;
-                lox = fminf(lox, X);
-                hix = fmaxf(hix, X);
-                loy = fminf(loy, Y);
-                hiy = fmaxf(hiy, Y);
-            }
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) {
-                lox = fminf(lox, __shfl_xor_sync(kFull, lox, o));
-                hix = fmaxf(hix, __shfl_xor_sync(kFull, hix, o));
-                loy = fminf(loy, __shfl_xor_sync(kFull, loy, o));
-                hiy = fmaxf(hiy, __shfl_xor_sync(kFull, hiy, o));
-            }
-            if (tid == 0) {  // centre cells floor(X + 1/2), one cell of stencil; 0.25 covers the FP32 error
-                s_box[0] = (int)floorf(lox + 0.25f) - 1;
-                s_box[1] = (int)floorf(loy + 0.25f) - 1;
-                s_box[2] = (int)floorf(hix + 0.75f) + 1;
-                s_box[3] = (int)floorf(hiy + 0.75f) + 1;
-            }
+            const int p0 = (int)blockIdx.x * P.group;
+            arc_box(p0, min(P.n_surface, p0 + P.group), P.n_surface, P.cx, P.cy, P.radius, tid, s_box);
         }
         __syncthreads();
         x0 = s_box[0];
@@ -221,47 +163,15 @@ __global__ void __launch_bounds__(kThreads) tile_steps_2d(TileArgs<S> P) {
             cell(0, lx, ly, f, c2, kc);
         }
     }
-    // A sampler's points, four lanes each (rho, Jx, Jy; the fourth repeats rho),
-    // in the last warps: the box's cells keep the first ones busy.
-    const int rt = kThreads - 1 - tid, quad = rt >> 2, comp = 3 - (rt & 3);
-    const int p0 = (int)blockIdx.x * P.group;
+    // A sampler's points, in the last warps: the box's cells keep the first ones busy.
+    const int rt = kThreads - 1 - tid, p0 = (int)blockIdx.x * P.group;
     const int n = sampler ? min(P.group, P.n_surface - p0) : 0;
     const bool warp_on = (rt >> 5) * 8 < n;  // whole warps sample (the shuffles)
-    const bool own = quad < n;
-    R w[9], n0 = R(0), n1 = R(0), acc = R(0);
-    int pc = 0;
-    if (SAMPLE && warp_on) {
-        const int p = p0 + (own ? quad : 0);
-        const int4 ctr = P.st_xyz[(long long)p * 9 + 4];
-        int lx = (ctr.x - x0) % nx, ly = (ctr.y - y0) % ny;  // the box is no larger than the lattice
-        lx += lx < 0 ? nx : 0;
-        ly += ly < 0 ? ny : 0;
-        pc = (min(max(ly, 1), th - 2) + H) * w0 + min(max(lx, 1), tw - 2) + H;  // in range by construction
-#pragma unroll
-        for (int l = 0; l < 9; ++l) w[l] = P.st_w[2 * ((long long)p * 9 + l) + (comp == 1 || comp == 2 ? 1 : 0)];
-        n0 = P.nrm[4 * (long long)p];
-        n1 = P.nrm[4 * (long long)p + 1];
-        acc = P.acc[5 * (long long)p + comp];
-    }
-    // lane 0: acc0 += p^2; lane 1: acc1 += u.u; lanes 2, 3: acc2, acc3 += u_a (u.n),
-    // the nine terms in the order of sample_point_2d_thread; acc4 stays zero (the
-    // terms of the third component are exact zeros)
-    auto sample = [&](int s) {
-        const R *m = mom + (size_t)(s & 1) * 3 * area + (size_t)(comp < 3 ? comp : 0) * area + pc;
-        R v[9];
-#pragma unroll
-        for (int l = 0; l < 9; ++l) v[l] = mul_rn(w[l], m[(l / 3 - 1) * w0 + l % 3 - 1]);
-        R sum = add_rn(add_rn(v[0], v[8]), v[4]);
-        sum = add_rn(sum, add_rn(v[2], v[6]));
-        sum = add_rn(sum, add_rn(add_rn(v[1], v[5]), add_rn(v[3], v[7])));
-        const int base = (tid & 31) & ~3;
-        const R pr = __shfl_sync(kFull, sum, base), u0 = __shfl_sync(kFull, sum, base + 1),
-                u1 = __shfl_sync(kFull, sum, base + 2);
-        const R a = mul_rn(u0, comp == 1 ? u0 : n0);
-        const R b = fma_rn(u1, comp == 1 ? u1 : n1, a);
-        const R x = comp == 0 ? pr : (comp == 1 ? R(1) : (comp == 2 ? u0 : u1));
-        acc = fma_rn(x, comp == 0 ? pr : b, acc);
-    };
+    const bool own = (rt >> 2) < n;
+    PointQuad<R> pt;
+    if (SAMPLE && warp_on)
+        pt.load(p0 + (own ? rt >> 2 : 0), 3 - (rt & 3), P.st_xyz, P.st_w, P.nrm, P.acc, x0, y0, tw, th, nx, ny, H, w0);
+    auto sample = [&](int s) { pt.add(mom + (size_t)(s & 1) * 3 * area, area, w0); };
     __syncthreads();
     for (int s = 1; s < k; ++s) {
         if (SAMPLE && warp_on) sample(s - 1);
@@ -284,7 +194,7 @@ __global__ void __launch_bounds__(kThreads) tile_steps_2d(TileArgs<S> P) {
     }
     if (SAMPLE && warp_on) {
         sample(k - 1);
-        if (own) P.acc[5 * (long long)(p0 + quad) + comp] = acc;
+        if (own) P.acc[5 * (long long)(p0 + (rt >> 2)) + pt.comp] = pt.acc;
     }
 }
 
@@ -303,17 +213,6 @@ cudaError_t allow_smem() {
         e = cudaFuncSetAttribute(tile_steps_2d<S, DRIVEN, SAMPLE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  optin - (int)fa.sharedSizeBytes);
     return e;
-}
-
-// Points per sampler CTA: an arc of at most kMaxArc cells, and no more points
-// than take about as long as a tile (FP64: the pipe needs 60 cycles per point
-// and step).
-template <typename S>
-int sampler_group(const Geometry &g) {
-    const double spacing = 6.283185307179586 * g.surface_radius / g.n_surface;
-    const int most = sizeof(typename Store<S>::R) == 8 ? 16 : kMaxGroup;
-    const int n = (int)std::fmin((double)most, (double)kMaxArc / spacing + 1.0);
-    return n < 1 ? 1 : n;
 }
 
 // What a step of the one-step kernels takes, in SM cycles (from measured steps
