@@ -132,6 +132,18 @@ struct RowBuf {
     float c2[c2_rows(C)][32 * C];
 };
 
+// Of `rows` rows from row y0 on (periodic in ny): the range [n0, n1) outside which
+// no row comes within `reach` rows of row c.
+__device__ __forceinline__ void near_rows(int c, int reach, int ny, int y0, int rows, int &n0, int &n1) {
+    n0 = 0;
+    n1 = rows;
+    if (rows > ny || 2 * reach + 1 >= ny) return;
+    const int d = ((c - y0) % ny + ny) % ny;  // the first image at or above y0, the one below it and above it
+    const bool below = d - ny + reach >= 0, own = d - reach < rows, above = d + ny - reach < rows;
+    n0 = below ? 0 : (own ? max(0, d - reach) : (above ? d + ny - reach : rows));
+    n1 = above ? rows : (own ? min(rows, d + reach + 1) : (below ? min(rows, d - ny + reach + 1) : 0));
+}
+
 // k = K steps of chunk rows [ya, yb) by one warp (warp-uniform flow).
 template <typename S, int C, int K>
 __device__ __forceinline__ void sweep(const BatchLat &L, int src, int chunk, int lane, RowBuf<S, C> &sm) {
@@ -160,8 +172,16 @@ __device__ __forceinline__ void sweep(const BatchLat &L, int src, int chunk, int
         const int x = (j * 32 + lane) * 4;
         xc[j] = x < wl ? ((x - H) % nx + nx) % nx : -1;
     }
-    // stage what step 1 of the it-th row (row y) reads: one commit group per row
+    // stage what step 1 of the it-th row reads: one commit group per row
     const int rows = yb - ya + 2 * (K - 1);
+    // Rows farther from the centre than the interface band hold fluid cells only
+    // and their c^2 is not read: FP32, 44 -> about 41 bytes per cell (512 x 192^2,
+    // 1000 points: 60.7 -> 58.5 ms).  FP16 is bound by instructions (57.8 -> 59.4
+    // ms), short rows by latency, and six levels of seven cells leave no registers.
+    constexpr bool kSkip = sizeof(S) == 4 && C >= 4 && C * steps_for(C) < 40;
+    const float c0sq = (float)(L.g.c0 * L.g.c0);
+    int near0 = 0, near1 = rows;
+    if (kSkip) near_rows(L.plan.ntile, L.plan.tx, ny, ya - (K - 1), rows, near0, near1);
     int ys = ((ya - (K - 1)) % ny + ny) % ny;  // row staged next
     auto stage = [&](int it) {
         if (it < rows) {
@@ -177,9 +197,17 @@ __device__ __forceinline__ void sweep(const BatchLat &L, int src, int chunk, int
                 copy_in(dst[3] + x, A + (3 * (size_t)nc + rm + xp[j]));
                 copy_in(dst[4] + x, A + (4 * (size_t)nc + rp + xp[j]));
             }
+            float *c2 = sm.c2[it & (CR - 1)] + lane * 4;
+            if (!kSkip || (it >= near0 && it < near1)) {
 #pragma unroll
-            for (int j = 0; j < PC; ++j)
-                if (xc[j] >= 0) copy_in(sm.c2[it & (CR - 1)] + (j * 32 + lane) * 4, c2f + (r0 + xc[j]));
+                for (int j = 0; j < PC; ++j)
+                    if (xc[j] >= 0) copy_in(c2 + j * 128, c2f + (r0 + xc[j]));
+            } else {
+#pragma unroll
+                for (int j = 0; j < PC; ++j)
+                    if ((j * 32 + lane) * 4 < 32 * C)
+                        *reinterpret_cast<float4 *>(c2 + j * 128) = make_float4(c0sq, c0sq, c0sq, c0sq);
+            }
             ys = ys == ny - 1 ? 0 : ys + 1;
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -442,6 +470,12 @@ bool plan_for(BatchLat *lats, int count, int rows_fixed) {
         lats[i].plan.nslab = 1;
         lats[i].plan.nseg = steps_for(c);
         lats[i].plan.H = sampler_group<S>(g);
+        // the object's centre row and the rows to either side that it and its
+        // interface band can reach (two more for rounding)
+        const double cy = g.center[1] - g.n[1] * std::floor(g.center[1] / g.n[1]);
+        lats[i].plan.ntile = cy >= 0.0 && cy < g.n[1] ? (int)cy : 0;
+        const double reach = std::sqrt(g.radius * g.radius + g.band_half) + 2.0;
+        lats[i].plan.tx = std::fabs(g.center[1]) < 1e9 && reach < g.n[1] ? (int)reach + 1 : g.n[1];
         if ((long long)count * box_groups(lats[i]) > 0x7fffffffll) return false;  // blocks of the sampler launch
     }
     int zc[9] = {0};
