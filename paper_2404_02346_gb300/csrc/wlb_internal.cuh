@@ -144,12 +144,12 @@ struct BatchTwoGroup {
     int cta_begin = 0, ctas = 0;  // its range of the CTA -> lattice table
 };
 // Choices of a batched two-step plan (the autotuner tries several):
-// z-chunks of about zc_target planes, slab heights capped at h_cap (0: the
-// tallest that fits), one_chunk: one 16-byte chunk per lane for every lattice
+// z-chunks of about zc_target planes (0: chosen with staging_warp by estimated
+// time), slab heights capped at h_cap (0: the tallest that fits), one_chunk: one 16-byte chunk per lane for every lattice
 // (rows over 32 vectors then take several warps) instead of two for wide rows;
 // staging_warp: a dedicated warp per CTA stages the planes.
 struct BatchTwoKnobs {
-    int zc_target = 32, h_cap = 0, one_chunk = 0, staging_warp = 0;
+    int zc_target = 0, h_cap = 0, one_chunk = 0, staging_warp = 0;
     int rows_2d = 0;  // 2D: rows per warp chunk (0: chosen to fill whole waves)
 };
 // Plans every lattice (its plan lands in lats[i].plan) and fills up to two

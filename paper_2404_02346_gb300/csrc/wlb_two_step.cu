@@ -1325,7 +1325,7 @@ bool plan_group(BatchLat *lats, const std::vector<int> &members, int smem_max, c
 }
 
 template <typename S>
-bool plan_batch_for(BatchLat *lats, int count, const BatchTwoKnobs &kn, BatchTwoGroup *groups, int *ngroups) {
+bool plan_batch_with(BatchLat *lats, int count, const BatchTwoKnobs &kn, BatchTwoGroup *groups, int *ngroups) {
     int dev = 0, smem_max = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
@@ -1350,6 +1350,61 @@ bool plan_batch_for(BatchLat *lats, int count, const BatchTwoKnobs &kn, BatchTwo
         }
     *ngroups = n;
     return true;
+}
+
+// Estimated time of a planned batch's launch, in us.  A CTA takes zc + 2 planes and
+// the latency of one and a half more to start and end; a plane takes its bytes at
+// the SM's share of the HBM rate, but no less than its chain of copies, barrier and
+// two steps, which a dedicated staging warp shortens.  Few CTAs of one size run in
+// whole waves of one per SM; else the SMs stay busy up to two thirds of the longest
+// CTA.  (Constants from 84 plans of each of eight batches, 4 x 160^3 to 64 lattices
+// of three sizes, FP32 and FP16: the choice was within 1.2 % of the fastest.)
+template <typename S>
+double batch_cost(const BatchLat *lats, int count, int sms) {
+    double work = 0, longest = 0;
+    long long ctas = 0;
+    for (int i = 0; i < count; ++i) {
+        const TwoStepPlan &pl = lats[i].plan;
+        const double bytes = (double)lats[i].g.n[0] * ((pl.H + 2) * (7.0 * sizeof(S) + 1.0) + pl.H * 7.0 * sizeof(S));
+        const double chain = pl.producer ? (sizeof(S) == 2 ? 1.47 : 1.89) : 1.95;
+        const double t = (pl.zc + 2) * std::max(chain, bytes / 43.9e3) + 1.5 * chain;
+        const int n = pl.nslab * pl.chunks;
+        work += n * t;
+        ctas += n;
+        longest = std::max(longest, t);
+    }
+    const double mean = work / (double)ctas;
+    if (longest <= 1.05 * mean && ctas <= 6ll * sms) return std::ceil((double)ctas / sms) * mean;
+    return work / sms + 0.66 * longest;
+}
+
+// The knobs as given, or with zc_target = 0 the z-chunks and staging of least
+// estimated time.  Measured, ms per run of three periods (z-chunks of 32 planes
+// staged by warp 0 -> this choice): 16 x 64^3 FP32 34.3 -> 20.3 (160 CTAs on 152
+// SMs before), 48 x 48^3 38.7 -> 24.8, 4 x 160^3 120 -> 86, 40 x 144^3 640 -> 575,
+// 32 of 96^3 / 160^3 FP16 439 -> 401, 64 of 96^3 / 128^3 / 160^3 758 -> 742.
+template <typename S>
+bool plan_batch_for(BatchLat *lats, int count, const BatchTwoKnobs &kn, BatchTwoGroup *groups, int *ngroups) {
+    if (kn.zc_target > 0) return plan_batch_with<S>(lats, count, kn, groups, ngroups);
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return false;
+    BatchTwoKnobs best = kn;
+    double best_cost = -1;
+    for (int sw = 0; sw < 2; ++sw)
+        for (int zc : {16, 24, 32, 48, 64, 96, 1 << 20}) {
+            BatchTwoKnobs k = kn;
+            k.zc_target = zc;
+            k.staging_warp = sw;
+            if (!plan_batch_with<S>(lats, count, k, groups, ngroups)) continue;
+            const double c = batch_cost<S>(lats, count, sms);
+            if (best_cost < 0 || c < best_cost) {
+                best_cost = c;
+                best = k;
+            }
+        }
+    return best_cost >= 0 && plan_batch_with<S>(lats, count, best, groups, ngroups);
 }
 
 // The groups' launches after the sampling launch: one after the other on s,
