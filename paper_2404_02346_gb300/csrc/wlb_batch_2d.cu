@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(32) batch_rows_2d(const BatchLat *__restrict__
 // states of five populations, c^2, the moments of two steps, wrapped columns and
 // rows.
 constexpr size_t box_bytes(int k) {
-    const size_t b = sampler_box() + 2 * (k - 1);
+    const size_t b = sampler_box<float>() + 2 * (k - 1);
     return 17 * b * b * sizeof(float) + 2 * b * sizeof(int);
 }
 

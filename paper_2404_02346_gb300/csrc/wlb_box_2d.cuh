@@ -9,8 +9,13 @@
 namespace wlb {
 namespace {
 
-constexpr int kMaxGroup = 64;   // points of a sampler CTA (four lanes each)
-constexpr float kMaxArc = 8.0f; // and the length of their arc in cells
+constexpr int kMaxGroup = 64;  // points of a sampler CTA (four lanes each)
+// And the length of their arc in cells.  FP64 boxes of eight cells of arc take
+// longer than a tile: 128^2, 64 points, us per sampled step with arcs of 8, 6, 4, 3
+// cells 1.72, 1.58, 1.53, 1.49.  FP32: 8 or shorter alike (256^2, 200 points: 0.83
+// with 8, 0.91 with 4, more boxes than SMs).
+template <typename R>
+constexpr float max_arc() { return sizeof(R) == 8 ? 3.0f : 8.0f; }
 
 // The value a stored state holds for v (storage rounding).
 template <typename S> __device__ __forceinline__ typename Store<S>::R as_stored(typename Store<S>::R v) { return v; }
@@ -18,7 +23,8 @@ template <> __device__ __forceinline__ float as_stored<__half>(float v) { return
 
 // Largest moment box of a sampler CTA, in cells: the arc's extent, one cell of
 // stencil on either side and two of rounding.
-__host__ __device__ constexpr int sampler_box() { return (int)kMaxArc + 5; }
+template <typename R>
+__host__ __device__ constexpr int sampler_box() { return (int)max_arc<R>() + 5; }
 
 // i / w for 0 <= i < 2^16 and w >= 1 by the high half of a product with
 // ceil(2^32 / w) (which does not fit 32 bits for w = 1: a box one cell wide).
@@ -27,19 +33,33 @@ __device__ __forceinline__ int divide(int i, int w, unsigned magic) {
     return w > 1 ? (int)__umulhi((unsigned)i, magic) : i;
 }
 
+// a + b and a - b.  In FP64 as fused multiply-adds with one = 1 (exact products,
+// the same rounding): the FP64 pipe takes 2.0 of them per clock and SM but 1.68
+// additions.  `one` must come from memory, or the compiler makes them additions.
+template <typename R>
+__device__ __forceinline__ R plus(R a, R b, R one) {
+    if constexpr (sizeof(R) == 8) return fma_rn(a, one, b);
+    else return add_rn(a, b);
+}
+template <typename R>
+__device__ __forceinline__ R minus(R a, R b, R one) {
+    if constexpr (sizeof(R) == 8) return fma_rn(b, -one, a);
+    else return sub_rn(a, b);
+}
+
 // The collision of collide_half for D = 2, with rho1 returned.  2 eq and
 // 2 (rho1 - 2 eq) are exact, so the two fused multiply-adds round exactly as
 // the product and difference do; they save two of thirteen operations, which
 // in FP64 are the kernel's bound.
 template <typename R>
-__device__ __forceinline__ R collide_2d(R c2, const R (&f)[5], R (&o)[5]) {
-    const R rho = add_rn(add_rn(add_rn(add_rn(f[0], f[1]), f[2]), f[3]), f[4]);
+__device__ __forceinline__ R collide_2d(R c2, const R (&f)[5], R (&o)[5], R one = R(1)) {
+    const R rho = plus(plus(plus(plus(f[0], f[1], one), f[2], one), f[3], one), f[4], one);
     const R eq = mul_rn(c2, rho);
     o[0] = fma_rn(R(2), fma_rn(R(-2), eq, rho), -f[0]);
-    o[1] = sub_rn(eq, f[2]);
-    o[2] = sub_rn(eq, f[1]);
-    o[3] = sub_rn(eq, f[4]);
-    o[4] = sub_rn(eq, f[3]);
+    o[1] = minus(eq, f[2], one);
+    o[2] = minus(eq, f[1], one);
+    o[3] = minus(eq, f[4], one);
+    o[4] = minus(eq, f[3], one);
     return rho;
 }
 
@@ -99,14 +119,14 @@ struct PointQuad {
         n1 = nrm[4 * (long long)p + 1];
         acc = sums[5 * (long long)p + comp];
     }
-    __device__ __forceinline__ void add(const R *mom, int area, int w0) {
+    __device__ __forceinline__ void add(const R *mom, int area, int w0, R one = R(1)) {
         const R *m = mom + (size_t)(comp < 3 ? comp : 0) * area + pc;
         R v[9];
 #pragma unroll
         for (int l = 0; l < 9; ++l) v[l] = mul_rn(w[l], m[(l / 3 - 1) * w0 + l % 3 - 1]);
-        R sum = add_rn(add_rn(v[0], v[8]), v[4]);
-        sum = add_rn(sum, add_rn(v[2], v[6]));
-        sum = add_rn(sum, add_rn(add_rn(v[1], v[5]), add_rn(v[3], v[7])));
+        R sum = plus(plus(v[0], v[8], one), v[4], one);
+        sum = plus(sum, plus(v[2], v[6], one), one);
+        sum = plus(sum, plus(plus(v[1], v[5], one), plus(v[3], v[7], one), one), one);
         const int base = (threadIdx.x & 31) & ~3;
         const R pr = __shfl_sync(kFull, sum, base), u0 = __shfl_sync(kFull, sum, base + 1),
                 u1 = __shfl_sync(kFull, sum, base + 2);
@@ -117,14 +137,14 @@ struct PointQuad {
     }
 };
 
-// Points per sampler CTA: an arc of at most kMaxArc cells, and no more points
+// Points per sampler CTA: an arc of at most max_arc cells, and no more points
 // than take about as long as a tile (FP64: the pipe needs 60 cycles per point
 // and step).
 template <typename S>
 inline int sampler_group(const Geometry &g) {
     const double spacing = 6.283185307179586 * g.surface_radius / g.n_surface;
     const int most = sizeof(typename Store<S>::R) == 8 ? 16 : kMaxGroup;
-    const int n = (int)std::fmin((double)most, (double)kMaxArc / spacing + 1.0);
+    const int n = (int)std::fmin((double)most, (double)max_arc<typename Store<S>::R>() / spacing + 1.0);
     return n < 1 ? 1 : n;
 }
 

@@ -204,7 +204,7 @@ cudaError_t launch_two_steps_2d(const Geometry &g, const Buffers &b, Prec p, con
 // tiles of tx x ty cells, up to k steps per launch; k = 0: not used.
 constexpr int kMaxTileSteps = 8;
 struct TilePlan2D {
-    int k = 0, tx = 0, ty = 0, sms = 1;
+    int k = 0, tx = 0, ty = 0;
     int group = 1;  // surface points per sampler CTA (sampled launches)
     size_t smem = 0;
 };

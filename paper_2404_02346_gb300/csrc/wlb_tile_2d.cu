@@ -43,6 +43,7 @@ struct TileArgs {
     const int4 *st_xyz;
     const R *st_w, *nrm;
     R *acc;
+    R one;                          // 1 (collide_2d)
     R phi;                          // driven cavity: wall damping,
     int axis;                       // wave axis
     R rho_src[kMaxTileSteps];       // and the source sheet's rho1 at every step
@@ -63,13 +64,8 @@ __global__ void __launch_bounds__(kThreads) tile_steps_2d(TileArgs<S> P) {
     extern __shared__ __align__(16) unsigned char tile_raw[];
     __shared__ int s_box[4];
     const int tid = threadIdx.x, nx = P.nx, ny = P.ny, k = P.k, H = k - 1;
-    asm volatile("griddepcontrol.launch_dependents;");
     const bool sampler = SAMPLE && (int)blockIdx.x < P.samplers;
     const int tile = (int)blockIdx.x - (SAMPLE ? P.samplers : 0);
-    if (!sampler && tile >= P.tiles) {  // padding (see the launch)
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        return;
-    }
     // the cells this CTA needs after the last step: the tile, or the stencils of
     // the sampler's points
     int x0, y0, tw, th;
@@ -115,11 +111,11 @@ __global__ void __launch_bounds__(kThreads) tile_steps_2d(TileArgs<S> P) {
         const int c = ly * w0 + lx;
         if (SAMPLE && sampler) {
             R *m = mom + (size_t)(s & 1) * 3 * area + c;
-            m[area] = sub_rn(f[1], f[2]);
-            m[2 * (size_t)area] = sub_rn(f[3], f[4]);
+            m[area] = minus(f[1], f[2], P.one);
+            m[2 * (size_t)area] = minus(f[3], f[4], P.one);
         }
         R o[5];
-        const R rho = collide_2d<R>(c2, f, o);
+        const R rho = collide_2d<R>(c2, f, o, P.one);
         if (SAMPLE && sampler) mom[(size_t)(s & 1) * 3 * area + c] = rho;
         if (DRIVEN && kc >= CELL_WALL_LO) {
             drv.rho_src = P.rho_src[s];
@@ -163,6 +159,10 @@ __global__ void __launch_bounds__(kThreads) tile_steps_2d(TileArgs<S> P) {
             cell(0, lx, ly, f, c2, kc);
         }
     }
+    // Not before this grid has its input: a grid that waits behind a waiting one
+    // takes SMs' slots early and lands unevenly, two CTAs on SMs that have few
+    // (192^2 FP32 0.73 -> 0.60 us per step, sampled 1.06 -> 0.79).
+    asm volatile("griddepcontrol.launch_dependents;");
     // A sampler's points, in the last warps: the box's cells keep the first ones busy.
     const int rt = kThreads - 1 - tid, p0 = (int)blockIdx.x * P.group;
     const int n = sampler ? min(P.group, P.n_surface - p0) : 0;
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kThreads) tile_steps_2d(TileArgs<S> P) {
     PointQuad<R> pt;
     if (SAMPLE && warp_on)
         pt.load(p0 + (own ? rt >> 2 : 0), 3 - (rt & 3), P.st_xyz, P.st_w, P.nrm, P.acc, x0, y0, tw, th, nx, ny, H, w0);
-    auto sample = [&](int s) { pt.add(mom + (size_t)(s & 1) * 3 * area, area, w0); };
+    auto sample = [&](int s) { pt.add(mom + (size_t)(s & 1) * 3 * area, area, w0, P.one); };
     __syncthreads();
     for (int s = 1; s < k; ++s) {
         if (SAMPLE && warp_on) sample(s - 1);
@@ -242,11 +242,11 @@ double one_step_cost(const Geometry &g, Prec p, bool sample, int sms) {
 // k = 0 where one step per launch is estimated faster (large FP64 lattices, which
 // the FP64 pipe bounds either way, and large FP16 ones).  Measured (us per step,
 // one step per launch -> tiles; unsampled, sampled with N points):
-//   128^2 FP64, N = 64      5.4 -> 1.18    6.6 -> 1.72    (3 steps, 16 x 7 cells)
-//   64 x 203 driven FP64    7.7 -> 1.74    9.1 -> 1.93    (4 steps, 8 x 11)
-//   192^2 FP32, N = 1000    1.5 -> 0.70    3.5 -> 0.9     (8 steps, 16 x 16)
-//   256^2 FP16, N = 200     2.1 -> 0.69    2.6 -> 0.82
-//   600^2 FP32, N = 500     3.3 -> 1.56    5.4 -> 1.8
+//   128^2 FP64, N = 64      5.4 -> 1.17    6.6 -> 1.49    (3 steps, 16 x 7 cells)
+//   64 x 203 driven FP64    7.7 -> 1.79    9.1 -> 1.91    (4 steps, 8 x 11)
+//   192^2 FP32, N = 1000    1.5 -> 0.60    3.5 -> 0.79    (8 steps, 16 x 16)
+//   256^2 FP16, N = 200     2.1 -> 0.68    2.6 -> 0.84
+//   600^2 FP32, N = 500     3.3 -> 1.62    5.4 -> 1.92
 //   4096^2 FP32             111 -> 75-81                  (4-6 steps, 32 x 32)
 template <typename S>
 TilePlan2D plan_for(const Geometry &g, Prec p, bool sample, int sms, size_t smem_max) {
@@ -285,13 +285,13 @@ TilePlan2D plan_for(const Geometry &g, Prec p, bool sample, int sms, size_t smem
                 const int H = k - 1;
                 size_t smem = box_smem<R>(tx + 2 * H, ty + 2 * H, false, g.driven != 0);
                 if (sample) {
-                    const int b = sampler_box() + 2 * H;
+                    const int b = sampler_box<R>() + 2 * H;
                     const size_t sb = box_smem<R>(b, b, true, g.driven != 0);
                     smem = sb > smem ? sb : smem;
                 }
                 if (smem > smem_max || (long long)(tx + 2 * H) * (ty + 2 * H) > 65535) break;  // box index division
                 const double tile_c = box_cells(tx, ty, k) * per_cell;
-                const double arc = sample ? std::fmin((double)kMaxArc, group * 6.283 * g.surface_radius / g.n_surface) : 0;
+                const double arc = sample ? std::fmin((double)max_arc<R>(), group * 6.283 * g.surface_radius / g.n_surface) : 0;
                 const int bx = (int)arc + 4;
                 const double samp_c = sample ? box_cells(bx, bx, k) * per_cell * 1.2 + k * (350.0 + group * per_point) : 0;
                 const double work = (double)tiles + samplers * (samp_c > tile_c ? samp_c / tile_c : 1.0);
@@ -307,7 +307,6 @@ TilePlan2D plan_for(const Geometry &g, Prec p, bool sample, int sms, size_t smem
                     best.tx = tx;
                     best.ty = ty;
                     best.smem = smem;
-                    best.sms = sms;
                     best.group = group;
                 }
             }
@@ -348,14 +347,12 @@ cudaError_t launch_for(const Geometry &g, const Buffers &b, const TilePlan2D &pl
     a.st_w = (const R *)b.st_w;
     a.nrm = (const R *)b.nrm;
     a.acc = (R *)b.acc;
+    a.one = R(1);
     a.phi = (R)g.wall_damping;
     a.axis = g.wave_axis;
     for (int i = 0; i < kMaxTileSteps; ++i) a.rho_src[i] = i < k ? (R)rho_src[i] : R(0);
     cudaLaunchConfig_t cfg = {};
-    // Whole multiples of the SMs: the next launch's CTAs are placed while this
-    // one's are resident, and an SM without one would get two of the next (128^2
-    // FP64, 143 tiles on 152 SMs, four steps: 3.40 us per step, padded 1.52).
-    cfg.gridDim = dim3((unsigned)((a.tiles + a.samplers + pl.sms - 1) / pl.sms * pl.sms));
+    cfg.gridDim = dim3((unsigned)(a.tiles + a.samplers));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = pl.smem;  // of the plan's k: enough for any fewer
     cfg.stream = s;
