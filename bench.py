@@ -503,7 +503,8 @@ def run_ensemble(args):
     rows2d = args.workload == "ensemble2d" and args.precision != "f64" and spl == 2
     if rows2d:
         spl = 6           # rows of 192 cells: six steps per launch
-        bpu = 2 * q * size + 4  # and c^2 read in place of the class byte
+        # no class byte; c^2 read for every row (FP16) or near the object only (FP32, not counted)
+        bpu = 2 * q * size + (4 if args.precision == "f16" else 0)
     launch_ms = tune["ms_per_step"] * spl
     achieved = bpu * cells_all / (launch_ms * 1e-3) / 1e9
     peaks = _peaks()

@@ -3,8 +3,8 @@
 //
 // Many lattices together are far larger than L2, so every launch streams all
 // populations through HBM and the bound is bytes per step: K steps per launch
-// cost 44 / K bytes per cell and step (FP32: five populations read and written,
-// c^2 read).  A warp owns a chunk of whole rows of one lattice and sweeps it
+// cost 40 / K bytes per cell and step (FP32: five populations read and written;
+// c^2 near the object comes on top).  A warp owns a chunk of whole rows of one lattice and sweeps it
 // once with K time levels in flight: when row p of step 1 is computed from the
 // staged populations, step l is computed on row p - l + 1 from the registers
 // that hold the previous rows of step l - 1.  Per level and cell that is five
@@ -22,8 +22,8 @@
 // Every step rounds its result to the storage type as a stored state would be
 // and the arithmetic per cell is that of the one-step kernels: the same bits.
 //
-// 512 lattices of 192 x 192 cells, FP32, six steps per launch: 142 us per launch,
-// 0.83 GB of HBM traffic (0.87 of the copy rate), against 3 x 155 us for two steps
+// 512 lattices of 192 x 192 cells, FP32, six steps per launch: 132 us per launch,
+// 0.76 GB of HBM traffic (0.84 of the copy rate), against 3 x 155 us for two steps
 // per launch; the samplers of 1000 points per lattice 107 us per launch against
 // 3 x 100 us for one thread per point with the steps recomputed per stencil cell.
 #include <algorithm>
