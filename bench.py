@@ -455,6 +455,7 @@ def run_ensemble(args):
     batch = wlb.Batch(probs, stream=stream)
     tune = batch.autotune(steps_per_trial=16)
     info = batch.info()
+    spl = batch.steps_per_launch(0)  # lattices of one width, or two steps each
     for _ in range(args.warmup):
         F = batch.run()
     torch.cuda.synchronize()
@@ -499,10 +500,8 @@ def run_ensemble(args):
     size = {"f32": 4, "f16": 2, "f64": 8}[args.precision]
     bpu = 2 * q * size + 1
     cells_all = sum(int(np.prod(p["n"][:p["dim"]])) for p in probs)
-    spl = info.steps_per_launch if info.steps_per_launch > 0 else 1
-    rows2d = args.workload == "ensemble2d" and args.precision != "f64" and spl == 2
+    rows2d = args.workload == "ensemble2d" and spl > 2  # row sweeps of several steps
     if rows2d:
-        spl = 6           # rows of 192 cells: six steps per launch
         # no class byte; c^2 read for every row (FP16) or near the object only (FP32, not counted)
         bpu = 2 * q * size + (4 if args.precision == "f16" else 0)
     launch_ms = tune["ms_per_step"] * spl
@@ -526,7 +525,7 @@ def run_ensemble(args):
         traffic = _traffic(_kernel_sha(2, "wlb_batch_2d.cu"), name="batch_rows_2d_d2q5_f32_ensemble512.md")
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": traffic, "kernel": "batched %supdate (%s storage), all lattices"
-                                          % ({1: "", 2: "two-step ", 6: "six-step "}[spl], args.precision),
+                                          % ("%d-step " % spl if spl > 1 else "", args.precision),
                 "bytes_per_cell_per_launch": bpu, "avg_launch_us": launch_ms * 1e3,
                 "peak_source": ("measured" if peaks and "hbm_gbs" in peaks else "fallback") + " hbm_gbs"}
     line = {

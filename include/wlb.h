@@ -137,9 +137,9 @@ typedef struct {
     int vector_path;            /* 1 if the row-vectorised update kernel is used */
     int steps_per_launch;       /* steps per update launch: 1, or 2 with
                                    wlb_set_two_step (the default for 3D
-                                   lattices where it applies); lattices that
-                                   report 1 may still take several steps per
-                                   launch in tiles (see wlb_step)               */
+                                   lattices where it applies); steps that
+                                   wlb_step takes in tiles are not counted
+                                   here (see wlb_get_launch_info)               */
     int two_step_rows;          /* slab height of the two-step kernel, 0 off    */
     int two_step_segments;      /* warps per lattice row (per x-tile) in it, 0 off */
     int two_step_tiles;         /* x-tiles per row in it (1: whole rows), 0 off */
@@ -366,7 +366,8 @@ typedef struct {
     int steps_per_launch;           /* 2: every launch advances all lattices two
                                        steps (wlb_set_two_step's kernel, one
                                        launch over every lattice's slabs) or
-                                       several (2D, wlb_batch_set_two_step)    */
+                                       several (2D: how many depends on the row
+                                       length, see wlb_batch_steps_per_launch) */
     int total_ctas;                 /* work units of that launch: blocks (3D)
                                        or warps, one per row chunk (2D); 0 if
                                        one step per launch                    */
@@ -378,6 +379,10 @@ wlb_status wlb_batch_create(const wlb_params *ps, int count, void *ws, size_t ws
 wlb_status wlb_batch_autotune(wlb_batch *b, int steps_per_trial, wlb_batch_tuning *best);
 wlb_status wlb_batch_run(wlb_batch *b, double *forces_out);
 wlb_status wlb_batch_get_info(const wlb_batch *b, wlb_batch_info *out);
+/* Steps that one launch of wlb_batch_run takes lattice `lattice` (0 .. count - 1)
+ * at most; a period's last launch takes what is left of it.  WLB_ERR_ARG for an
+ * index out of range. */
+wlb_status wlb_batch_steps_per_launch(const wlb_batch *b, int lattice, int *steps);
 /* Steps two per launch for the whole batch: on by default when all run
  * lengths, windows and periods are even and every lattice is periodic and
  * either 3D with FP32/FP16 rows the two-step slab kernel takes (then one
@@ -455,6 +460,17 @@ wlb_status wlb_mlp_destroy(wlb_mlp *m);
 
 /* Sizes and counters of a handle. */
 wlb_status wlb_get_info(const wlb_handle *h, wlb_info *out);
+
+/* How wlb_step advances the lattice with the present settings: one update
+ * launch of unsampled ([0]) and of sampled ([1]) steps. */
+typedef struct {
+    int steps[2];               /* steps it takes at most                       */
+    int tile[2][3];             /* extent of its overlapped tiles in cells, zeros
+                                   where it takes no such tiles                 */
+    int sampler_blocks;         /* blocks that sample the surface for a sampled
+                                   launch of tiles, 0 without such launches     */
+} wlb_launch_info;
+wlb_status wlb_get_launch_info(const wlb_handle *h, wlb_launch_info *out);
 
 /* Steps two per launch: the update of Eqs. (62)-(64), (71) applied twice in
  * one kernel, bit-identical to two single steps.  Each block owns a slab of

@@ -63,6 +63,15 @@ class Info(ctypes.Structure):
     ]
 
 
+class LaunchInfo(ctypes.Structure):
+    """Mirror of ``wlb_launch_info``."""
+    _fields_ = [
+        ("steps", ctypes.c_int * 2),
+        ("tile", (ctypes.c_int * 3) * 2),
+        ("sampler_blocks", ctypes.c_int),
+    ]
+
+
 class BatchTuning(ctypes.Structure):
     """Mirror of ``wlb_batch_tuning``."""
     _fields_ = [("threads_per_block", ctypes.c_int), ("blocks_per_sm", ctypes.c_int),
@@ -103,6 +112,7 @@ _SIGNATURES = {
     "wlb_save_state": (ctypes.c_int, [_VP, _VP, ctypes.c_size_t]),
     "wlb_load_state": (ctypes.c_int, [_VP, _VP, ctypes.c_size_t]),
     "wlb_get_info": (ctypes.c_int, [_VP, ctypes.POINTER(Info)]),
+    "wlb_get_launch_info": (ctypes.c_int, [_VP, ctypes.POINTER(LaunchInfo)]),
     "wlb_set_two_step": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_int]),
     "wlb_set_two_step_tiles": (ctypes.c_int, [_VP, ctypes.c_int]),
     "wlb_set_two_step_staging": (ctypes.c_int, [_VP, ctypes.c_int]),
@@ -116,6 +126,7 @@ _SIGNATURES = {
     "wlb_batch_autotune": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.POINTER(BatchTuning)]),
     "wlb_batch_run": (ctypes.c_int, [_VP, _DP]),
     "wlb_batch_get_info": (ctypes.c_int, [_VP, ctypes.POINTER(BatchInfo)]),
+    "wlb_batch_steps_per_launch": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]),
     "wlb_batch_set_two_step": (ctypes.c_int, [_VP, ctypes.c_int]),
     "wlb_batch_last_error": (ctypes.c_char_p, [_VP]),
     "wlb_batch_destroy": (ctypes.c_int, [_VP]),
@@ -247,6 +258,12 @@ class Solver:
         _check(lib().wlb_get_info(self._h, ctypes.byref(out)), self._h, "wlb_get_info")
         return out
 
+    def launch_info(self):
+        """Steps per update launch, tiles and sampler blocks (wlb_get_launch_info)."""
+        out = LaunchInfo()
+        _check(lib().wlb_get_launch_info(self._h, ctypes.byref(out)), self._h, "wlb_get_launch_info")
+        return out
+
     def init(self):
         _check(lib().wlb_init(self._h), self._h, "wlb_init")
 
@@ -375,6 +392,13 @@ class Batch:
         out = BatchInfo()
         self._bcheck(lib().wlb_batch_get_info(self._h, ctypes.byref(out)), "wlb_batch_get_info")
         return out
+
+    def steps_per_launch(self, lattice=0):
+        """Steps one launch takes a lattice at most (wlb_batch_steps_per_launch)."""
+        out = ctypes.c_int()
+        self._bcheck(lib().wlb_batch_steps_per_launch(self._h, int(lattice), ctypes.byref(out)),
+                     "wlb_batch_steps_per_launch")
+        return out.value
 
     def set_two_step(self, enable=True):
         """Two steps per launch for the whole batch (wlb_batch_set_two_step)."""

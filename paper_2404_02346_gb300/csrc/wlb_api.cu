@@ -629,6 +629,20 @@ wlb_status wlb_get_info(const wlb_handle *h, wlb_info *out) {
     return WLB_OK;
 }
 
+wlb_status wlb_get_launch_info(const wlb_handle *h, wlb_launch_info *out) {
+    if (!h || !out) return WLB_ERR_ARG;
+    *out = wlb_launch_info{};
+    for (int s = 0; s < 2; ++s) {
+        const int k = tile_steps(h, s != 0);
+        out->steps[s] = h->two_step ? 2 : (k > 0 ? k : 1);
+        if (k == 0) continue;
+        const int t2[3] = {h->tile[s].tx, h->tile[s].ty, 1}, t3[3] = {h->tile3.tx, h->tile3.ty, h->tile3.tz};
+        for (int a = 0; a < 3; ++a) out->tile[s][a] = h->g.dim == 2 ? t2[a] : t3[a];
+        if (s == 1) out->sampler_blocks = h->g.dim == 2 ? wlb::tile_samplers(h->g, h->tile[1]) : h->tile3.boxes;
+    }
+    return WLB_OK;
+}
+
 wlb_status wlb_destroy(wlb_handle *h) {
     if (!h) return WLB_ERR_ARG;
     DeviceGuard dg(h->device);

@@ -944,6 +944,12 @@ wlb_status wlb_batch_get_info(const wlb_batch *b, wlb_batch_info *out) {
     return WLB_OK;
 }
 
+wlb_status wlb_batch_steps_per_launch(const wlb_batch *b, int lattice, int *steps) {
+    if (!b || !steps || lattice < 0 || lattice >= b->count) return WLB_ERR_ARG;
+    *steps = !b->two ? 1 : (b->rows2d ? b->lat[(size_t)lattice].plan.nseg : 2);
+    return WLB_OK;
+}
+
 wlb_status wlb_batch_set_two_step(wlb_batch *b, int enable) {
     if (!b) return WLB_ERR_ARG;
     if (enable && !b->two_ok) return bfail(b, WLB_ERR_ARG, "two steps per launch not available for this batch");

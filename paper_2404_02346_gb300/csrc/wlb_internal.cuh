@@ -208,6 +208,8 @@ struct TilePlan2D {
     int group = 1;  // surface points per sampler CTA (sampled launches)
     size_t smem = 0;
 };
+// Sampler CTAs of a sampled launch.
+inline int tile_samplers(const Geometry &g, const TilePlan2D &pl) { return (g.n_surface + pl.group - 1) / pl.group; }
 // out[0] for unsampled, out[1] for sampled launches.
 cudaError_t plan_tile_2d(const Geometry &g, Prec p, TilePlan2D out[2]);
 // k <= pl.k steps from buffer src into src ^ 1, the first at step index t_mod of

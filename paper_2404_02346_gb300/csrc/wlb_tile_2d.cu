@@ -339,7 +339,7 @@ cudaError_t launch_for(const Geometry &g, const Buffers &b, const TilePlan2D &pl
     a.k = k;
     a.n_surface = g.n_surface;
     a.group = pl.group;
-    a.samplers = sample ? (g.n_surface + pl.group - 1) / pl.group : 0;
+    a.samplers = sample ? tile_samplers(g, pl) : 0;
     a.cx = (float)g.center[0];
     a.cy = (float)g.center[1];
     a.radius = (float)g.surface_radius;
