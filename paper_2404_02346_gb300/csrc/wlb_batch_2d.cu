@@ -328,9 +328,7 @@ __global__ void __launch_bounds__(kBoxThreads) batch_sample_boxes_2d(const Batch
     const size_t nc = (size_t)L.g.ncell;
     const S *__restrict__ A = (const S *)L.b.pop[n & 1];
     const float *__restrict__ c2f = (const float *)L.b.c2;
-    if (tid < 32)
-        arc_box(p0, min(np, p0 + group), np, (float)L.g.center[0], (float)L.g.center[1], (float)L.g.surface_radius,
-                tid, s_box);
+    if (tid < 32) arc_box(p0, min(np, p0 + group), np, circle_of(L.g), tid, s_box);
     __syncthreads();
     const int x0 = s_box[0], y0 = s_box[1], tw = s_box[2] - x0 + 1, th = s_box[3] - y0 + 1;
     const int w0 = tw + 2 * H, h0 = th + 2 * H, area = w0 * h0;
@@ -459,7 +457,7 @@ bool plan_for(BatchLat *lats, int count, int rows_fixed) {
     int tallest[9] = {0};
     for (int i = 0; i < count; ++i) {
         const Geometry &g = lats[i].g;
-        if (g.dim != 2 || g.driven || g.ncell > (1ll << 28)) return false;
+        if (g.dim != 2 || g.driven || g.ncell > (1ll << 28) || !boxes_fit(g)) return false;
         const int c = cells_per_lane<S>(g.n[0]);
         if (c == 0) return false;
         rows_of[c] += g.n[1];

@@ -63,15 +63,36 @@ __device__ __forceinline__ R collide_2d(R c2, const R (&f)[5], R (&o)[5], R one 
     return rho;
 }
 
+// Circle of the surface points: whole cells of its centre and the rest, so that
+// the FP32 positions below are relative to the centre.  On an absolute axis their
+// spacing reaches half a cell at 2^22 cells and stencils would leave their box.
+struct Circle {
+    int x, y;
+    float fx, fy, radius;
+};
+__host__ __device__ inline Circle circle_of(const Geometry &g) {
+    const double x = floor(g.center[0]), y = floor(g.center[1]);
+    return Circle{(int)x, (int)y, (float)(g.center[0] - x), (float)(g.center[1] - y), (float)g.surface_radius};
+}
+
+// Whether box coordinates and their differences fit 32 bits; sampled steps of
+// other lattices go without boxes.
+inline bool boxes_fit(const Geometry &g) {
+    constexpr int kMost = 1 << 29;
+    for (int a = 0; a < 2; ++a)
+        if (g.n[a] > kMost || !(std::fabs(g.center[a]) <= kMost)) return false;
+    return true;
+}
+
 // Extent of the cells that the stencils of points p0 .. p1 - 1 of the circle
-// read, by one warp: b = first column, first row, last column, last row.
-__device__ __forceinline__ void arc_box(int p0, int p1, int n_surface, float cx, float cy, float radius, int lane,
-                                        int *b) {
+// read, by one warp: b = first column, first row, last column, last row (not
+// wrapped).
+__device__ __forceinline__ void arc_box(int p0, int p1, int n_surface, const Circle &c, int lane, int *b) {
     float lox = 1e30f, hix = -1e30f, loy = 1e30f, hiy = -1e30f;
     for (int p = p0 + lane; p < p1; p += 32) {
         float sn, cs;
         sincospif((float)(2 * p + 1) / (float)n_surface, &sn, &cs);
-        const float X = cx + radius * cs, Y = cy + radius * sn;
+        const float X = c.fx + c.radius * cs, Y = c.fy + c.radius * sn;
         lox = fminf(lox, X);
         hix = fmaxf(hix, X);
         loy = fminf(loy, Y);
@@ -84,11 +105,15 @@ __device__ __forceinline__ void arc_box(int p0, int p1, int n_surface, float cx,
         loy = fminf(loy, __shfl_xor_sync(kFull, loy, o));
         hiy = fmaxf(hiy, __shfl_xor_sync(kFull, hiy, o));
     }
-    if (lane == 0) {  // centre cells floor(X + 1/2), one cell of stencil; 0.25 covers the FP32 error
-        b[0] = (int)floorf(lox + 0.25f) - 1;
-        b[1] = (int)floorf(loy + 0.25f) - 1;
-        b[2] = (int)floorf(hix + 0.75f) + 1;
-        b[3] = (int)floorf(hiy + 0.75f) + 1;
+    // centre cells floor(X + 1/2), one cell of stencil; 0.25 covers the FP32 error:
+    // 2^-24 radius (2 pi for the angle, 3 for the sine, its product and the sum),
+    // and twice 2 pi more beyond 2^23 points, is below 0.1 for radii up to 2^16
+    // (the lattice of a larger circle takes over 400 GB)
+    if (lane == 0) {
+        b[0] = c.x + (int)floorf(lox + 0.25f) - 1;
+        b[1] = c.y + (int)floorf(loy + 0.25f) - 1;
+        b[2] = c.x + (int)floorf(hix + 0.75f) + 1;
+        b[3] = c.y + (int)floorf(hiy + 0.75f) + 1;
     }
 }
 

@@ -39,7 +39,7 @@ struct TileArgs {
     long long ncell;
     int tx, ty, tiles_x, tiles, k;
     int n_surface, group, samplers;  // points, points per sampler CTA, sampler CTAs (the first blocks)
-    float cx, cy, radius;           // circle of the surface points
+    Circle circle;                  // of the surface points
     const int4 *st_xyz;
     const R *st_w, *nrm;
     R *acc;
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kThreads) tile_steps_2d(TileArgs<S> P) {
     if (sampler) {
         if (tid < 32) {
             const int p0 = (int)blockIdx.x * P.group;
-            arc_box(p0, min(P.n_surface, p0 + P.group), P.n_surface, P.cx, P.cy, P.radius, tid, s_box);
+            arc_box(p0, min(P.n_surface, p0 + P.group), P.n_surface, P.circle, tid, s_box);
         }
         __syncthreads();
         x0 = s_box[0];
@@ -255,6 +255,7 @@ TilePlan2D plan_for(const Geometry &g, Prec p, bool sample, int sms, size_t smem
     const double per_cell = kDouble ? 8.0 : (sizeof(S) == 2 ? 1.1 : 0.95);
     const double per_point = kDouble ? 60.0 : 6.0;
     const int nx = g.n[0], ny = g.n[1];
+    if (sample && !boxes_fit(g)) return TilePlan2D{};
     const int group = sample ? sampler_group<S>(g) : 0;
     const int samplers = sample ? (g.n_surface + group - 1) / group : 0;
     auto box_cells = [](int w, int h, int k) {
@@ -340,9 +341,7 @@ cudaError_t launch_for(const Geometry &g, const Buffers &b, const TilePlan2D &pl
     a.n_surface = g.n_surface;
     a.group = pl.group;
     a.samplers = sample ? tile_samplers(g, pl) : 0;
-    a.cx = (float)g.center[0];
-    a.cy = (float)g.center[1];
-    a.radius = (float)g.surface_radius;
+    a.circle = circle_of(g);
     a.st_xyz = b.st_xyz;
     a.st_w = (const R *)b.st_w;
     a.nrm = (const R *)b.nrm;
