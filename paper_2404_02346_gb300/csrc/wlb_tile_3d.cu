@@ -352,10 +352,11 @@ __global__ void __launch_bounds__(kSampleThreads) sample_boxes(SampleArgs<S> a, 
     R(*mom)[4][kMomCells] = reinterpret_cast<R(*)[4][kMomCells]>(box_raw + sizeof(R) * 7 * kMomCells);  // rho, J at t, t+1
     const Geometry &g = a.g;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2], tid = threadIdx.x;
+    // the grid is an upper bound: only entry 0 exists for every block
+    if ((int)blockIdx.x >= aux(a.st_xyz, 0)) return;  // block-uniform
     const long long e = 1 + 5 * (long long)blockIdx.x;
-    const int boxes = aux(a.st_xyz, 0), bx = aux(a.st_xyz, e), by = aux(a.st_xyz, e + 1), bz = aux(a.st_xyz, e + 2),
+    const int bx = aux(a.st_xyz, e), by = aux(a.st_xyz, e + 1), bz = aux(a.st_xyz, e + 2),
               first = aux(a.st_xyz, e + 3), count = aux(a.st_xyz, e + 4);
-    if ((int)blockIdx.x >= boxes) return;  // block-uniform
     auto wrap = [](int v, int n) {
         v %= n;
         return v < 0 ? v + n : v;
@@ -472,7 +473,7 @@ __global__ void __launch_bounds__(kSampleThreads) sample_boxes(SampleArgs<S> a, 
 // ---------------------------------------------------------------- host side: plans and launches
 
 // Boxes that can hold a centre cell: those the sphere's surface, one cell thick
-// on either side, passes through.
+// on either side, passes through, and no more than there are points.
 int count_boxes(const Geometry &g) {
     const double R = g.surface_radius;
     int n = 0;
@@ -492,7 +493,7 @@ int count_boxes(const Geometry &g) {
                 }
                 n += near <= R * R && far >= R * R;
             }
-    return n;
+    return n < g.n_surface ? n : g.n_surface;
 }
 
 template <typename S>
