@@ -1047,11 +1047,14 @@ wlb_status wlb_mlp_train(wlb_mlp *m, const float *x, const float *t, long long n
         MLP_CUDA(m, cudaMalloc(&m->perm, sizeof(int) * n), "permutation buffer");
         m->perm_cap = n;
     }
-    std::vector<int> perm((size_t)n);
+    // two orders in turn: a copy from pageable memory may still read the one it
+    // was given while the epoch runs; the synchronisation at its end frees it
+    std::vector<int> orders[2];
     uint64_t s = seed;
     const long long nb = n / batch;  // whole batches per epoch
     if (nb < 1) return WLB_ERR_ARG;
-    auto shuffle = [&] {
+    for (int i = 0; i < (epochs > 1 ? 2 : 1); ++i) orders[i].resize((size_t)n);
+    auto shuffle = [&](std::vector<int> &perm) {
         for (long long i = 0; i < n; ++i) perm[(size_t)i] = (int)i;
         for (long long i = n - 1; i > 0; --i) {  // Fisher-Yates
             const long long j = (long long)(splitmix(s) % (uint64_t)(i + 1));
@@ -1061,9 +1064,10 @@ wlb_status wlb_mlp_train(wlb_mlp *m, const float *x, const float *t, long long n
         }
     };
     MLP_CUDA(m, prepare_train(m), "pack");
-    shuffle();
+    shuffle(orders[0]);
     for (int ep = 0; ep < epochs; ++ep) {
-        MLP_CUDA(m, cudaMemcpyAsync(m->perm, perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, m->stream), "perm");
+        MLP_CUDA(m, cudaMemcpyAsync(m->perm, orders[ep & 1].data(), sizeof(int) * n, cudaMemcpyHostToDevice, m->stream),
+                 "perm");
         MLP_CUDA(m, cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream), "zero loss");
         const float lr_e = lr * std::pow(lr_final / lr, (float)ep / (float)(epochs > 1 ? epochs - 1 : 1));
         // train_weights refreshes the training copies itself, the others not
@@ -1074,7 +1078,7 @@ wlb_status wlb_mlp_train(wlb_mlp *m, const float *x, const float *t, long long n
             const float c2 = 1.0f / (1.0f - std::pow(0.999f, (float)m->adam_t));
             MLP_CUDA(m, train_step(m, x, t, m->perm, k * batch, batch, nullptr, lr_e, c1, c2), "training step");
         }
-        if (ep + 1 < epochs) shuffle();  // while this epoch runs (its order is on the device)
+        if (ep + 1 < epochs) shuffle(orders[(ep + 1) & 1]);  // while this epoch runs
         float l = 0;
         MLP_CUDA(m, cudaMemcpyAsync(&l, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream), "loss");
         wlb_status st = check_err(m);
