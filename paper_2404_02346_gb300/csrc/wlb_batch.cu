@@ -416,6 +416,17 @@ int rows_steps(const wlb_batch *b) {
     return k;
 }
 
+// Steps that the first n launches take, a mean over the cells of all lattices:
+// launches of different widths and a period's last one differ in steps.
+double rows_steps_taken(const wlb_batch *b, int n) {
+    double steps = 0, cells = 0;
+    for (const BatchLat &L : b->lat) {
+        steps += (double)L.g.ncell * (double)wlb::batch2d_steps_taken(L, n);
+        cells += (double)L.g.ncell;
+    }
+    return steps / cells;
+}
+
 cudaError_t issue_steps(wlb_batch *b, int nsteps, int threads, int bps, cudaStream_t s) {
     const int grid = b->n_sm * bps;
     if (b->two) {  // step counts are even in this mode
@@ -755,7 +766,9 @@ wlb_status wlb_batch_autotune(wlb_batch *b, int steps_per_trial, wlb_batch_tunin
         // time one plan: a warm-up pair of steps, then steps from step 0 (all
         // lattices active)
         const int per_launch = b->rows2d ? rows_steps(b) : 2;
-        const int launches = (steps_per_trial + per_launch - 1) / per_launch, steps = launches * per_launch;
+        int launches = steps_per_trial / per_launch + (steps_per_trial % per_launch != 0);
+        if (b->rows2d) launches = std::min(launches, b->turns.launches);  // later ones find every lattice done
+        const double steps = b->rows2d ? rows_steps_taken(b, launches) : 2.0 * launches;
         auto trial = [&](float *ms) -> cudaError_t {
             if (b->rows2d) {
                 cudaError_t e = issue_rows(b, 0, 1);
@@ -770,7 +783,7 @@ wlb_status wlb_batch_autotune(wlb_batch *b, int steps_per_trial, wlb_batch_tunin
             if (e == cudaSuccess) e = issue_steps(b, 2, b->threads, b->blocks_per_sm, b->stream);
             if (e == cudaSuccess) e = cudaMemsetAsync(b->d_step, 0, sizeof(long long), b->stream);
             if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
-            if (e == cudaSuccess) e = issue_steps(b, steps, b->threads, b->blocks_per_sm, b->stream);
+            if (e == cudaSuccess) e = issue_steps(b, 2 * launches, b->threads, b->blocks_per_sm, b->stream);
             if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
             if (e == cudaSuccess) e = cudaEventElapsedTime(ms, e0, e1);
@@ -834,7 +847,7 @@ wlb_status wlb_batch_autotune(wlb_batch *b, int steps_per_trial, wlb_batch_tunin
         if (best) {
             best->threads_per_block = b->two_threads;
             best->blocks_per_sm = 1;
-            best->ms_per_step = best_ms / steps;
+            best->ms_per_step = (float)(best_ms / steps);
             best->z_chunk = b->dim == 3 ? best_kn.zc_target : b->lat[0].plan.zc;
             best->slab_rows_cap = b->dim == 3 ? best_kn.h_cap : 0;
             best->one_chunk_per_lane = b->dim == 3 ? best_kn.one_chunk : 0;

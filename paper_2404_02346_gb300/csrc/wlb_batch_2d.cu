@@ -579,6 +579,12 @@ BatchTurns batch2d_turns(const BatchLat *lats, int count) {
     return r;
 }
 
+long long batch2d_steps_taken(const BatchLat &L, int n) {
+    const long long per = launches_per_period(L);
+    const long long t = n / per * L.period + std::min(L.period, n % per * L.plan.nseg);
+    return std::min(L.n_steps, t);
+}
+
 cudaError_t launch_batch2d_rows(Prec p, const BatchTwoGroup *groups, int ngroups, const BatchLat *lats,
                                 const int *task_lat, const int *task_first, int count, const BatchTurns &turns, int n,
                                 cudaStream_t s) {

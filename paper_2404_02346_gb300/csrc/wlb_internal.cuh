@@ -185,6 +185,8 @@ struct BatchTurns {
     int launches = 0, first_sampled = 0, groups = 0, steps = 0;
 };
 BatchTurns batch2d_turns(const BatchLat *lats, int count);
+// Steps of a planned lattice in the first n launches of a run.
+long long batch2d_steps_taken(const BatchLat &L, int n);
 // Launch n of a run: every lattice that is not done advances by the steps its
 // period has left, plan.nseg at most; the state before it is in buffer n & 1.
 cudaError_t launch_batch2d_rows(Prec p, const BatchTwoGroup *groups, int ngroups, const BatchLat *lats,
