@@ -38,6 +38,7 @@ constexpr int kDepth = 2;       // rows of populations staged ahead
 constexpr int kMaxSteps = 8;
 constexpr int kMaxRows = 128;   // rows per warp chunk
 constexpr int kMinRows = 8;
+constexpr long long kMaxLaunches = 1ll << 28;  // of a run: launch and step-in-period numbers fit 32 bits
 constexpr int kBoxThreads = 256;
 
 // Steps per launch of rows with C cells per lane: about as many as 255 registers
@@ -467,6 +468,7 @@ bool plan_for(BatchLat *lats, int count, int rows_fixed) {
         lats[i].plan.threads = 32;
         lats[i].plan.nslab = 1;
         lats[i].plan.nseg = steps_for(c);
+        if (lats[i].n_steps / lats[i].period > kMaxLaunches / launches_per_period(lats[i])) return false;
         lats[i].plan.H = sampler_group<S>(g);
         // the object's centre row and the rows to either side that it and its
         // interface band can reach (two more for rounding)
