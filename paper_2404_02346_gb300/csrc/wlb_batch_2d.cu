@@ -27,6 +27,7 @@
 // per launch; the samplers of 1000 points per lattice 107 us per launch against
 // 3 x 100 us for one thread per point with the steps recomputed per stencil cell.
 #include <algorithm>
+#include <map>
 #include <type_traits>
 
 #include "wlb_box_2d.cuh"
@@ -454,15 +455,13 @@ bool plan_for(BatchLat *lats, int count, int rows_fixed) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return false;
     double slots[9] = {0};  // warps of the launch that the device holds
-    long long rows_of[9] = {0};
-    int tallest[9] = {0};
+    std::map<int, long long> heights[9];  // lattices by height: an ensemble has few (512 of one: 0.2 ms less to create)
     for (int i = 0; i < count; ++i) {
         const Geometry &g = lats[i].g;
         if (g.dim != 2 || g.driven || g.ncell > (1ll << 28) || !boxes_fit(g)) return false;
         const int c = cells_per_lane<S>(g.n[0]);
         if (c == 0) return false;
-        rows_of[c] += g.n[1];
-        tallest[c] = std::max(tallest[c], g.n[1]);
+        ++heights[c][g.n[1]];
         lats[i].plan = TwoStepPlan{};
         lats[i].plan.chunks_per_lane = c;
         lats[i].plan.threads = 32;
@@ -480,7 +479,7 @@ bool plan_for(BatchLat *lats, int count, int rows_fixed) {
     }
     int zc[9] = {0};
     for (int c = 2; c <= 8; ++c) {
-        if (rows_of[c] == 0) continue;
+        if (heights[c].empty()) continue;
         int bps = 0;
         cudaError_t e = with_cells<S>(c, [&](auto cc) {
             constexpr int C = decltype(cc)::value;
@@ -498,11 +497,10 @@ bool plan_for(BatchLat *lats, int count, int rows_fixed) {
             for (int z = kMaxRows; z >= kMinRows; --z) {
                 long long t = 0;
                 int tall = 0;  // rows of the longest chunk
-                for (int i = 0; i < count; ++i) {
-                    if (lats[i].plan.chunks_per_lane != c) continue;
-                    const int n = (lats[i].g.n[1] + z - 1) / z;
-                    t += n;
-                    tall = std::max(tall, (lats[i].g.n[1] + n - 1) / n);
+                for (const auto &[ny, lattices] : heights[c]) {
+                    const int n = (ny + z - 1) / z;
+                    t += n * lattices;
+                    tall = std::max(tall, (ny + n - 1) / n);
                 }
                 const double cost = std::ceil((double)t / slots[c]) * (tall + 2 * (steps_for(c) - 1) + 2);
                 if (rows <= 0 || cost < best) {
