@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kBoxThreads) batch_sample_boxes_2d(const Batch
     const size_t nc = (size_t)L.g.ncell;
     const S *__restrict__ A = (const S *)L.b.pop[n & 1];
     const float *__restrict__ c2f = (const float *)L.b.c2;
-    if (tid < 32) arc_box(p0, min(np, p0 + group), np, circle_of(L.g), tid, s_box);
+    if (tid < 32) arc_box(p0, min(np, p0 + group), np, L.circle, tid, s_box);
     __syncthreads();
     const int x0 = s_box[0], y0 = s_box[1], tw = s_box[2] - x0 + 1, th = s_box[3] - y0 + 1;
     const int w0 = tw + 2 * H, h0 = th + 2 * H, area = w0 * h0;
@@ -469,6 +469,7 @@ bool plan_for(BatchLat *lats, int count, int rows_fixed) {
         lats[i].plan.nseg = steps_for(c);
         if (lats[i].n_steps / lats[i].period > kMaxLaunches / launches_per_period(lats[i])) return false;
         lats[i].plan.H = sampler_group<S>(g);
+        lats[i].circle = circle_of(g);
         // the object's centre row and the rows to either side that it and its
         // interface band can reach (two more for rounding)
         const double cy = g.center[1] - g.n[1] * std::floor(g.center[1] / g.n[1]);

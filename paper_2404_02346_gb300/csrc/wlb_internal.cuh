@@ -117,6 +117,15 @@ struct SideStream {
 cudaError_t launch_two_steps(const Geometry &g, const Buffers &b, Prec p, const TwoStepPlan &pl, int src, bool sample,
                              int *err, cudaStream_t s, const SideStream &side);
 
+// Circle of a 2D lattice's surface points for the box samplers (wlb_box_2d.cuh):
+// whole cells of its centre and the rest, so that FP32 positions are relative to
+// the centre.  On an absolute axis their spacing reaches half a cell at 2^22
+// cells and stencils would leave their box.
+struct Circle {
+    int x = 0, y = 0;
+    float fx = 0, fy = 0, radius = 0;
+};
+
 // One lattice of a batched ensemble (wlb_batch.cu): geometry, buffers, its
 // protocol lengths and, when the batch runs two steps per launch, its plan.
 struct BatchLat {
@@ -124,6 +133,7 @@ struct BatchLat {
     Buffers b;
     long long n_steps, window_begin, period;
     TwoStepPlan plan;
+    Circle circle;  // with the plan of plan_batch2d_rows
 };
 
 // The setup (launch_setup) of all lattices of a batch in three launches; lats
