@@ -439,7 +439,7 @@ wlb_status wlb_batch_destroy(wlb_batch *b);
  *                        tensor memory and the weights streamed from L2.
  *   wlb_mlp_set_fused    fused = 1 (default): predict as above; 0: one
  *                        tensor-core GEMM launch per layer through device
- *                        memory in batch_max chunks (the training forward).
+ *                        memory in batch_max chunks (the fused path's check).
  *                        Both give the same bits.  WLB_ERR_ARG otherwise.
  * All calls synchronise the stream before returning.  WLB_ERR_TIMEOUT if a
  * tensor-core completion wait gave up (the kernel returns instead of hanging).

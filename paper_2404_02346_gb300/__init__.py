@@ -492,7 +492,7 @@ class MLP:
 
     def set_fused(self, fused):
         """True (default): predict with the one-launch fused network; False:
-        one GEMM launch per layer (the training forward)."""
+        one GEMM launch per layer (the fused network's check)."""
         self._mcheck(lib().wlb_mlp_set_fused(self._h, 1 if fused else 0), "wlb_mlp_set_fused")
 
     def predict(self, x):

@@ -14,10 +14,11 @@
 //
 // A lane owns C consecutive cells of the row, so that one shuffle per direction
 // and level moves a row by one cell; rows of C V cells wrap around by the
-// shuffle's lane, others are staged with a halo of at least K - 1 columns on
-// either side whose results are dropped.  Rows travel through shared memory:
-// 16-byte asynchronous copies in (kDepth rows ahead, c^2 kept for all levels),
-// bulk copies out.
+// shuffle's lane, others are staged with a halo of at least K columns on either
+// side, for every step spoils one more column from the ends of the staged row, and
+// their results are dropped.  Rows travel through shared memory: 16-byte
+// asynchronous copies in (kDepth rows ahead, c^2 kept for all levels), 16-byte
+// streaming stores out.
 //
 // Every step rounds its result to the storage type as a stored state would be
 // and the arithmetic per cell is that of the one-step kernels: the same bits.
@@ -50,8 +51,8 @@ __host__ __device__ constexpr int steps_for(int c) { return c <= 4 ? 8 : (c <= 7
 // Rows of c^2 kept: kDepth ahead, steps - 1 behind.
 __host__ __device__ constexpr int c2_rows(int c) { return c <= 4 ? 16 : 8; }
 // Halo columns staged on either side of a row that its lanes do not cover exactly:
-// at least steps - 1, a whole number of 16-byte pieces.
-__host__ __device__ constexpr int halo_for(int c, int w) { return (steps_for(c) - 1 + w - 1) / w * w; }
+// at least a column per step, a whole number of 16-byte pieces.
+__host__ __device__ constexpr int halo_for(int c, int w) { return (steps_for(c) + w - 1) / w * w; }
 
 // Step t of a lattice at launch n and the steps of that launch: whole periods of
 // launches of plan.nseg steps, the last one of a period shorter, so that a period's

@@ -86,6 +86,10 @@ bool update_is_vectorised(const Geometry &g, Prec p);
 // segments of one warp each.  Slab height H, slabs and z-chunks of the grid,
 // segments per row (per x-tile when rows are split into ntile tiles of tx
 // cells), chunks per lane, block size and dynamic shared memory.
+// The 2D sweeps keep their plans in the same fields: zc rows per warp chunk and
+// chunks of them.  batch_rows_2d (wlb_batch_2d.cu) besides: chunks_per_lane cells
+// per lane, nseg steps per launch, H points per sampler block, ntile the row of the
+// object's centre and tx the rows to either side of it that its band can reach.
 struct TwoStepPlan {
     int H = 0, nslab = 0, chunks = 0, zc = 0, nseg = 0, chunks_per_lane = 0, threads = 0;
     int ntile = 1, tx = 0;  // x-tiles per row and their width (1: whole rows)

@@ -247,7 +247,7 @@ double one_step_cost(const Geometry &g, Prec p, bool sample, int sms) {
 //   192^2 FP32, N = 1000    1.5 -> 0.60    3.5 -> 0.79    (8 steps, 16 x 16)
 //   256^2 FP16, N = 200     2.1 -> 0.68    2.6 -> 0.84
 //   600^2 FP32, N = 500     3.3 -> 1.62    5.4 -> 1.92
-//   4096^2 FP32             111 -> 75-81                  (4-6 steps, 32 x 32)
+//   4096^2 FP32             111 -> 75-81                  (4 steps, 70 x 57)
 template <typename S>
 TilePlan2D plan_for(const Geometry &g, Prec p, bool sample, int sms, size_t smem_max) {
     using R = typename Store<S>::R;
