@@ -99,8 +99,8 @@ HOST_MARKER = b"// -------------------------------------------------------------
 def _kernel_sha(steps_per_launch=1, two_step_src="wlb_two_step.cu"):
     """sha256 over the update kernel's device code and the device header it
     includes: wlb_step.cu whole, or the two-step source (wlb_two_step.cu, or
-    wlb_two_step_2d.cu for the 2D batches) up to its host-side part (plans and
-    launches, which a profile's counters do not depend on)."""
+    wlb_two_step_2d.cu or wlb_batch_2d.cu for the 2D batches) up to its host-side
+    part (plans and launches, which a profile's counters do not depend on)."""
     csrc = os.path.join(ROOT, "paper_2404_02346_gb300", "csrc")
     h = hashlib.sha256()
     if steps_per_launch == 2:
@@ -110,6 +110,8 @@ def _kernel_sha(steps_per_launch=1, two_step_src="wlb_two_step.cu"):
     else:
         h.update(open(os.path.join(csrc, "wlb_step.cu"), "rb").read())
     h.update(open(os.path.join(csrc, "wlb_kernels.cuh"), "rb").read())
+    if two_step_src == "wlb_batch_2d.cu":
+        h.update(open(os.path.join(csrc, "wlb_box_2d.cuh"), "rb").read())  # its collision
     return h.hexdigest()
 
 
