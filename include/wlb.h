@@ -183,7 +183,8 @@ wlb_status wlb_init(wlb_handle *h);
  * take up to eight steps of overlapped tiles, where that is estimated faster
  * than one (periodic or driven, any row length; bit-identical), and on 3D
  * lattices without wlb_set_two_step (FP32 and FP16 rows of whole 16-byte
- * vectors, periodic or driven) two.  WLB_ERR_STATE before wlb_init. */
+ * vectors that are not whole warps of them, periodic or driven) two;
+ * wlb_get_launch_info tells which.  WLB_ERR_STATE before wlb_init. */
 wlb_status wlb_step(wlb_handle *h, long long n_steps, int sample);
 
 /* Time-averaged force from the samples taken since wlb_init, Eq. (14) in
